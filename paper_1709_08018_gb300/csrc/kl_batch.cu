@@ -54,7 +54,7 @@ __global__ void batch_parts_kernel(const GroupDesc* __restrict__ D,
 
 __global__ void batch_combine_kernel(const GroupDesc* __restrict__ D,
                                      const uint32_t* __restrict__ bases, uint32_t n,
-                                     uint32_t total, int mixed, unsigned long long* fb,
+                                     uint32_t total, int mixed, int filter, unsigned long long* fb,
                                      uint32_t* fb_count) {
   for (uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total;
        idx += gridDim.x * blockDim.x) {
@@ -62,40 +62,37 @@ __global__ void batch_combine_kernel(const GroupDesc* __restrict__ D,
     const Plan L = D[g].L;
     const View V = D[g].V;
     const Tables T = D[g].T;
-    combine_entry(V, L, D[g].ptol, mixed, idx - bases[g], T, g, fb, fb_count);
+    combine_entry(V, L, D[g].ptol, mixed, idx - bases[g], T, g, fb, fb_count, filter != 0);
   }
 }
 
-// One persistent launch for the whole batch.  Queue order: all groups' FP64
-// fallback units (32 per item; mixed mode only), then every group's items in
+// One persistent launch for a whole mixed batch.  Queue order: all groups' FP64
+// fallback units (32 per item), then every group's items in
 // group order.  Counters are published per group whenever a warp moves to
-// another group (the item, hence the group, is uniform over the warp, and
-// over the block for FP64 items).
+// another group (the item, hence the group, is uniform over the warp).
 // Registers are capped at 48 (10 blocks of 128 threads per SM): the group
 // lookup and descriptor spill at the single render's 40, and the batch ran
 // 3% faster at 48.
-template <int BT, bool MIXED>
-__global__ void __launch_bounds__(BT, 1280 / BT) batch_render_kernel(
+template <int BT>
+__global__ void __launch_bounds__(BT, 1280 / BT) batch_mixed_kernel(
     const GroupDesc* __restrict__ D, const uint32_t* __restrict__ item_bases, uint32_t n,
     uint32_t n_items, const unsigned long long* __restrict__ fb,
     const uint32_t* __restrict__ fb_count, uint32_t cmax, uint32_t* queue) {
-  // mixed items are drawn per warp (32 prefixes each, no block barrier), FP64
-  // items per block (BT prefixes)
-  constexpr uint32_t IT = MIXED ? 32u : (uint32_t)BT;
-  const uint32_t fb_units = MIXED ? 3u * cmax * (*fb_count) : 0u;
-  const uint32_t n64 = (fb_units + IT - 1) / IT;
+  // items are drawn per warp (32 prefixes each, no block barrier)
+  const uint32_t fb_units = 3u * cmax * (*fb_count);
+  const uint32_t n64 = (fb_units + 31u) / 32u;
   const uint32_t total = n64 + n_items;
   Tally t;
   uint32_t words = 0;
   int gcur = -1;
   // the current group's items are [glo, ghi): consecutive items of a warp
-  // (or block) usually stay in one group, which then needs no search
+  // usually stay in one group, which then needs no search
   uint32_t glo = 0u, ghi = 0u;  // empty: the first item searches
   for (;;) {
-    const uint32_t item = MIXED ? next_item_warp(queue) : next_item(queue);
+    const uint32_t item = next_item_warp(queue);
     if (item >= total) break;
-    if (MIXED && item < n64) {
-      const uint32_t unit = item * IT + (threadIdx.x & 31u);
+    if (item < n64) {
+      const uint32_t unit = item * 32u + (threadIdx.x & 31u);
       if (unit < fb_units) {
         const unsigned long long ent = fb[unit / (3u * cmax)];
         const uint32_t rem = unit % (3u * cmax);
@@ -128,12 +125,44 @@ __global__ void __launch_bounds__(BT, 1280 / BT) batch_render_kernel(
     const View V = D[g].V;
     const Tables T = D[g].T;
     const Work Wk = D[g].Wk;
-    if (MIXED)
-      mixed_item<32>(local - glo, Wk, L, V, T, t, words, D[g].img);
-    else
-      fp64_item<BT>(local - glo, Wk, L, V, T, t, words, D[g].img);
+    mixed_item<32>(local - glo, Wk, L, V, T, t, words, D[g].img);
   }
   if (gcur >= 0) publish_counts(t.in_window, words, 0, t.atomics, D[gcur].cnt);
+}
+
+// One persistent launch for a whole FP64 batch: warps take items (32 prefixes x
+// one suffix chunk of one group) in group order.  A warp that moves to another
+// group first finishes the one it leaves (its undecided words) and publishes
+// that group's counts.  The groups share the view.
+template <int BT>
+__global__ void __launch_bounds__(BT, 1024 / BT) batch_words_kernel(
+    const GroupDesc* __restrict__ D, View V, const uint32_t* __restrict__ item_bases, uint32_t n,
+    uint32_t n_items, uint32_t* queue) {
+  __shared__ WarpQueue s_queue[BT / 32];
+  __shared__ ExactCtx s_ctx[BT / 32];
+  const uint32_t wi = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  ExactCtx& C = s_ctx[wi];
+  WordWarp<KL_FP64> w(&C, &s_queue[wi]);
+  int gcur = -1;
+  // the current group's items are [glo, ghi): consecutive items of a warp
+  // usually stay in one group, which then needs no search
+  uint32_t glo = 0u, ghi = 0u;  // empty: the first item searches
+  for (;;) {
+    const uint32_t item = next_item_warp(queue);
+    if (item >= n_items) break;
+    if (item - glo >= ghi - glo) {  // outside [glo, ghi): another group
+      const int g = (int)find_group(item_bases, n, item);
+      if (gcur >= 0) w.finish(D[gcur].cnt);
+      gcur = g;
+      glo = item_bases[g];
+      ghi = item_bases[g + 1];
+      if (lane == 0) C = {D[g].T, V, D[g].L.ns, D[g].L.npairs, D[g].img};
+      __syncwarp();
+    }
+    const GroupDesc& d = D[gcur];
+    word_item(w, item - glo, d.Wk, d.L, V, C.T, C.img);
+  }
+  if (gcur >= 0) w.finish(D[gcur].cnt);
 }
 
 // Culling disks and prefix norms of every group (culled batches): unit =
@@ -229,32 +258,31 @@ const void* render_fn(int bt, bool mixed, bool cull) {
   }
   if (mixed) {
     switch (bt) {
-      case 64: return (const void*)batch_render_kernel<64, true>;
-      case 256: return (const void*)batch_render_kernel<256, true>;
-      default: return (const void*)batch_render_kernel<128, true>;
+      case 64: return (const void*)batch_mixed_kernel<64>;
+      case 256: return (const void*)batch_mixed_kernel<256>;
+      default: return (const void*)batch_mixed_kernel<128>;
     }
   }
   switch (bt) {
-    case 64: return (const void*)batch_render_kernel<64, false>;
-    case 256: return (const void*)batch_render_kernel<256, false>;
-    default: return (const void*)batch_render_kernel<128, false>;
+    case 64: return (const void*)batch_words_kernel<64>;
+    case 256: return (const void*)batch_words_kernel<256>;
+    default: return (const void*)batch_words_kernel<128>;
   }
 }
 
 template <int BT>
 void launch_batch(int grid, cudaStream_t s, bool mixed, bool cull, const GroupDesc* D,
-                  const uint32_t* item_bases, uint32_t n, uint32_t n_items,
+                  const View& V, const uint32_t* item_bases, uint32_t n, uint32_t n_items,
                   const unsigned long long* fb, uint32_t* cnt2, uint32_t cmax) {
+  uint32_t* queue = cnt2 + 1;
   if (cull && mixed)
-    batch_cull_kernel<BT, true><<<grid, BT, 0, s>>>(D, item_bases, n, n_items, cnt2 + 1);
+    batch_cull_kernel<BT, true><<<grid, BT, 0, s>>>(D, item_bases, n, n_items, queue);
   else if (cull)
-    batch_cull_kernel<BT, false><<<grid, BT, 0, s>>>(D, item_bases, n, n_items, cnt2 + 1);
+    batch_cull_kernel<BT, false><<<grid, BT, 0, s>>>(D, item_bases, n, n_items, queue);
   else if (mixed)
-    batch_render_kernel<BT, true><<<grid, BT, 0, s>>>(D, item_bases, n, n_items, fb, cnt2, cmax,
-                                                      cnt2 + 1);
+    batch_mixed_kernel<BT><<<grid, BT, 0, s>>>(D, item_bases, n, n_items, fb, cnt2, cmax, queue);
   else
-    batch_render_kernel<BT, false><<<grid, BT, 0, s>>>(D, item_bases, n, n_items, fb, cnt2, cmax,
-                                                       cnt2 + 1);
+    batch_words_kernel<BT><<<grid, BT, 0, s>>>(D, V, item_bases, n, n_items, queue);
 }
 
 bool same_frame(const kl_params& a, const kl_params& b) {
@@ -320,7 +348,7 @@ int enqueue(kl_batch* b, uint32_t* images, uint64_t* counters, void* ws, cudaStr
   if (check_launch() != KL_OK) return KL_ECUDA;
   const uint32_t gc = (b->n_comb + 127) / 128;
   batch_combine_kernel<<<gc < 1048576u ? gc : 1048576u, 128, 0, s>>>(
-      D, bases + (n + 1), n, b->n_comb, b->mixed, fb, cnt2);
+      D, bases + (n + 1), n, b->n_comb, b->mixed, !b->mixed && !b->cull, fb, cnt2);
   if (check_launch() != KL_OK) return KL_ECUDA;
   if (b->cull) {
     const uint32_t gd = (b->n_disk + 3) / 4;  // four warps per block
@@ -331,17 +359,19 @@ int enqueue(kl_batch* b, uint32_t* images, uint64_t* counters, void* ws, cudaStr
   const uint32_t* item_bases = bases + 2 * (n + 1);
   const int grid = b->sms * b->occ;
   const bool cull = b->cull != 0;
+  const View V = make_view(&b->params[0]);  // shared by the groups
   switch (b->bt) {
     case 64:
-      launch_batch<64>(grid, s, b->mixed, cull, D, item_bases, n, b->n_items, fb, cnt2, b->cmax);
+      launch_batch<64>(grid, s, b->mixed, cull, D, V, item_bases, n, b->n_items, fb, cnt2,
+                       b->cmax);
       break;
     case 256:
-      launch_batch<256>(grid, s, b->mixed, cull, D, item_bases, n, b->n_items, fb, cnt2,
-                        b->cmax);
+      launch_batch<256>(grid, s, b->mixed, cull, D, V, item_bases, n, b->n_items, fb, cnt2,
+                       b->cmax);
       break;
     default:
-      launch_batch<128>(grid, s, b->mixed, cull, D, item_bases, n, b->n_items, fb, cnt2,
-                        b->cmax);
+      launch_batch<128>(grid, s, b->mixed, cull, D, V, item_bases, n, b->n_items, fb, cnt2,
+                       b->cmax);
   }
   return check_launch();
 }
@@ -398,9 +428,8 @@ extern "C" int kl_batch_create(const kl_params* params, uint32_t n_groups, kl_ba
       return st;
     }
     // culled: warp items of 32 prefixes x one top-level block
-    b->works[g] = b->cull    ? make_work(L, 32, L.cnb[L.clev - 1], 1, 1u)
-                  : b->mixed ? make_work(L, 32, L.npairs, 1, chunk)
-                             : make_work(L, b->bt, L.ns, 1, 2u * chunk);
+    b->works[g] = b->cull ? make_work(L, 32, L.cnb[L.clev - 1], 1, 1u)
+                          : make_work(L, 32, L.npairs, 1, chunk);
     b->bases[g] = (uint32_t)parts;
     b->bases[(n_groups + 1) + g] = (uint32_t)comb;
     b->bases[2 * (n_groups + 1) + g] = (uint32_t)items;

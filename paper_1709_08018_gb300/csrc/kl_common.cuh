@@ -44,6 +44,8 @@ constexpr uint32_t kNearPar = 2u;    // |tr^2 - 4 det| small: near-parabolic (cu
 constexpr uint32_t kWide = 4u;       // local FP32 frame unsafe (far or huge offsets)
 constexpr uint32_t kFallback = 8u;   // KL_MIXED, KL_DF64: words of this prefix run in FP64
 constexpr uint32_t kDfRange = 16u;   // a pole-form constant outside the double-float range
+constexpr uint32_t kNoFilter = 32u;  // no filter constants: words take the exact map (kl_filter.cuh)
+constexpr uint32_t kOnFp32 = 64u;    // KL_MIXED: words on the FP32 map (its record is pre32's)
 
 // FP64 fallback work unit: a chunk of this many suffix points.
 constexpr uint32_t kFbChunk = 64;
@@ -73,6 +75,7 @@ struct View {
   double x0, y1, sx, sy;
   uint32_t W, H;
   uint32_t hiW, hiH;  // high words of (double)W and (double)H
+  float kappa, ik;    // sy / sx and sx / sy
 };
 
 struct Group {
@@ -96,6 +99,16 @@ struct __align__(16) Pre32 {
 struct __align__(16) PreDF {
   float h[8], l[8];
 };
+
+// Filter constants of one prefix (kl_filter.cuh).
+struct __align__(16) PreF {
+  float k1, k2, g1, g2;    // k = k1 + i k2, g = g1 + i g2
+  float axf, ayf, eb, c0;  // alpha in the local frame (row units 1/kappa); 32 eps |g|; c0
+  int axi, ayi;            // integer part of alpha's pixel coordinates (0 for a far alpha)
+  float rg;                // 1 / |g|
+  int pad;
+};
+static_assert(sizeof(PreF) <= sizeof(Pre32), "filter constants take the FP32 record's place");
 
 // Disk bounding one culling block of suffix points (FP64 points).
 struct __align__(16) Disk64 {
@@ -437,21 +450,191 @@ __device__ void part_entry(const Group& G, const Plan& L, int renorm, uint32_t i
   }
 }
 
+constexpr float kEps24 = 0x1p-24f;
+
+// FP64 compares and conversions run on the FP64 pipe (2 lanes per SM); where
+// the bits decide, the integer pipe takes them instead.
+__device__ __forceinline__ uint32_t abs_hi(double d) {
+  return (uint32_t)__double2hiint(d) & 0x7FFFFFFFu;
+}
+// |d| < lim (lim finite and positive)
+__device__ __forceinline__ bool abs_below(double d, double lim) {
+  const uint32_t a = abs_hi(d), b = abs_hi(lim);
+  return a < b || (a == b && (uint32_t)__double2loint(d) < (uint32_t)__double2loint(lim));
+}
+// d rounded to nearest even, as (float)d; normal results on the integer pipe.
+__device__ __forceinline__ float f32_of(double d) {
+  const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
+  const uint32_t e = (hi & 0x7FFFFFFFu) - 0x38100000u;  // biased exponent 897 and up ...
+  if (e >= 0x0FD00000u) return (float)d;                // ... below 1150, else the conversion
+  const uint32_t m = __funnelshift_l(lo, (hi & 0x7FFFFFFFu) - 0x38000000u, 3);
+  const uint32_t rem = lo & 0x1FFFFFFFu;
+  const uint32_t up = rem > 0x10000000u || (rem == 0x10000000u && (m & 1u)) ? 1u : 0u;
+  return __uint_as_float((m + up) | (hi & 0x80000000u));
+}
+// f as a double
+__device__ __forceinline__ double f64_of(float f) {
+  const uint32_t b = __float_as_uint(f), a = b & 0x7FFFFFFFu;
+  if (a - 0x00800000u >= 0x7F000000u) return (double)f;  // zero, denormal, not finite
+  return __hiloint2double((int)((b & 0x80000000u) | ((a >> 3) + 0x38000000u)), (int)(a << 29));
+}
+// floor of |d| < 2^31 as a double, and as an integer
+__device__ __forceinline__ double floor_int(double d, int& i) {
+  const double magic = 6755399441055744.0;  // 1.5 2^52: the integer in the low word
+  const double t = __dadd_rd(d, magic);
+  i = __double2loint(t);
+  return __dsub_rn(t, magic);
+}
+
 // A double as a double-float: hi = fl32(d), lo = fl32(d - hi).
 __device__ __forceinline__ void split_df(double d, float& hi, float& lo) {
-  hi = __double2float_rn(d);
-  lo = __double2float_rn(d - (double)hi);
+  hi = f32_of(d);
+  lo = f32_of(d - f64_of(hi));
+}
+
+// Filter constants of a prefix in pole form: gamma, alpha's pixel coordinates
+// (ax, ay) and sx beta = (c1, c2).  false: a constant outside the range in
+// which the bound holds (no word may then be certified).
+__device__ __forceinline__ bool filter_consts(const View& V, const Pre64& c, PreF& f) {
+  const float b1 = f32_of(c.c1), b2 = f32_of(c.c2), gr = f32_of(c.gr), gi = f32_of(c.gi);
+  const float q = __frcp_rn(fmaf(b1, b1, b2 * b2));
+  f.k1 = b1 * q;
+  f.k2 = -b2 * q;
+  f.g1 = fmaf(f.k1, gr, -(f.k2 * gi));
+  f.g2 = fmaf(f.k1, gi, f.k2 * gr);
+  // a near alpha: integer part and fraction; a far one (deep zooms): as it is
+  double fx = 0.0, fy = 0.0;
+  f.axi = f.ayi = 0;
+  if (abs_below(c.ax, 1048576.0) && abs_below(c.ay, 1048576.0)) {  // 2^20
+    fx = floor_int(c.ax, f.axi);
+    fy = floor_int(c.ay, f.ayi);
+  }
+  f.axf = f32_of(c.ax - fx);
+  f.ayf = f32_of(c.ay - fy) * V.ik;
+  const float ag = fabsf(f.g1) + fabsf(f.g2), ak = fabsf(f.k1) + fabsf(f.k2);
+  f.eb = 32.0f * kEps24 * ag;
+  f.c0 = 4.0f * kEps24 * (2.0f + 2.0f * V.ik + fabsf(f.axf) + fabsf(f.ayf));
+  f.rg = fminf(__frcp_rn(ag), 1e12f);
+  f.pad = 0;
+  // k's range keeps |w|^2 of a certified word clear of FP32 underflow and
+  // overflow in the exact map's own FP32 steps (gamma near 0: |w| is not tied
+  // to |gamma|)
+  const float kmax = fabsf(gr) + fabsf(gi) > 1e-12f ? 1e17f : 1e12f;
+  return ak > 1e-12f && ak < kmax && ag < 1e17f && fabsf(f.axf) < 1e30f &&
+         fabsf(f.ayf) < 1e30f && V.ik > 1e-6f && V.ik < 1e6f;
+}
+
+// The filter constants of a slot lie in its FP32 record, which prefixes on the
+// FP64 or double-float map do not read.
+__device__ __forceinline__ PreF* filter_slot(const Tables& T, uint32_t slot) {
+  return reinterpret_cast<PreF*>(T.pre32 + slot);
+}
+
+// Everything the words of one prefix need.
+struct PrefixRec {
+  Pre64 c64;
+  Pre32 c32;  // KL_MIXED, not kFallback
+  PreDF cd;   // KL_DF64, not kDirect
+  uint32_t fl;
+};
+
+// |tr^2 - 4 det| < ptol max(1, |tr|^2), exactly as in FP64.  An FP32 estimate
+// (error below 4e-6 of |tr|^2 + 4 |det|: six roundings and the two conversions)
+// settles all but the closest cases.
+__device__ __forceinline__ bool near_parabolic(const dc& tr, const dc& det, double ptol) {
+  const float a = f32_of(tr.re), b = f32_of(tr.im), c = f32_of(det.re), d = f32_of(det.im);
+  const float t2f = fmaf(a, a, b * b);
+  const float qr = fmaf(a, a, -(b * b)) - 4.0f * c, qi = 2.0f * a * b - 4.0f * d;
+  const float q = sqrtf(fmaf(qr, qr, qi * qi)), lim = (float)ptol * fmaxf(1.0f, t2f);
+  const float err = 4e-6f * (t2f + 4.0f * (fabsf(c) + fabsf(d))) + 1e-6f * lim;
+  if (q - lim > err && q < 1e18f) return false;
+  const dc tr2m4 = csub(cmul(tr, tr), {4.0 * det.re, 4.0 * det.im});
+  const double t2 = tr.re * tr.re + tr.im * tr.im;
+  const double lim2 = ptol * fmax(1.0, t2);
+  return tr2m4.re * tr2m4.re + tr2m4.im * tr2m4.im < lim2 * lim2;
+}
+
+// Prefix slot r of last letter x: the matrix P = H L and its constants.
+__device__ __forceinline__ void prefix_rec(const View& V, const Plan& L, double ptol, int prec,
+                                           const Tables& T, int x, uint32_t r, PrefixRec& R) {
+  const bool mixed = prec == KL_MIXED, df = prec == KL_DF64;
+  const PartM& TL = T.Lt[(uint32_t)x * L.p3_q1 + r / L.p3_pq];
+  const M2 P = L.p > L.q ? mmul(T.Ht[(uint32_t)TL.edge * L.p3_pq + r % L.p3_pq], TL.m) : TL.m;
+  const dc det = mdet(P);
+  uint32_t fl = 0;
+  if (mixed && near_parabolic(cadd(P.p, P.s), det, ptol)) fl |= kNearPar;
+  Pre64& c64 = R.c64;
+  // |P10| > 1e-12 of the largest entry: exponents within 2^-37 settle it
+  const uint32_t er = max(abs_hi(P.r.re), abs_hi(P.r.im)) >> 20;
+  const uint32_t em = max(max(max(abs_hi(P.p.re), abs_hi(P.p.im)),
+                              max(abs_hi(P.q.re), abs_hi(P.q.im))),
+                          max(max(abs_hi(P.s.re), abs_hi(P.s.im)), er << 20)) >> 20;
+  bool pole = er + 37u >= em && em < 2047u && er > 0u;
+  if (!pole) {
+    const double scale = fmax(fmax(cabs1(P.p), cabs1(P.q)), fmax(cabs1(P.r), cabs1(P.s)));
+    pole = cabs1(P.r) > 1e-12 * scale;
+  }
+  if (!pole) {
+    fl |= kDirect;
+    c64 = {P.p.re, P.p.im, P.q.re, P.q.im, P.r.re, P.r.im, P.s.re, P.s.im};
+  } else {
+    const dc inv10 = crcp(P.r);
+    const dc alpha = cmul(P.p, inv10);
+    const dc gamma = cmul(P.s, inv10);
+    const dc mbeta = cmul(det, cmul(inv10, inv10));  // -beta
+    const double ax = (alpha.re - V.x0) * V.sx;
+    const double ay = (V.y1 - alpha.im) * V.sy;
+    const double c1 = -V.sx * mbeta.re, c2 = -V.sx * mbeta.im;
+    const double c3 = V.sy * mbeta.im, c4 = -V.sy * mbeta.re;
+    c64 = {gamma.re, gamma.im, ax, ay, c1, c2, c3, c4};
+    const double lim = 1048576.0;  // 2^20
+    if (!(abs_below(ax, lim) && abs_below(ay, lim) && abs_below(gamma.re, 1e15) &&
+          abs_below(gamma.im, 1e15)))
+      fl |= kWide;
+  }
+  if (df) {
+    // the double-float constants; a constant (nonzero) outside [1e-30, 1e30]
+    // would leave the float range in the per-word products
+    const double cv[8] = {c64.gr, c64.gi, c64.ax, c64.ay, c64.c1, c64.c2, c64.c3, c64.c4};
+    for (int q = 0; q < 8; ++q) {
+      split_df(cv[q], R.cd.h[q], R.cd.l[q]);
+      if (!abs_below(cv[q], 1e30) || (cv[q] != 0.0 && abs_below(cv[q], 1e-30))) fl |= kDfRange;
+    }
+  }
+  if ((mixed && (fl & (kDirect | kNearPar | kWide))) ||
+      (df && (fl & (kDirect | kWide | kDfRange))))
+    fl |= kFallback;
+  if (mixed && !(fl & kFallback)) {
+    fl |= kOnFp32;
+    int axi, ayi;
+    const double fx = floor_int(c64.ax, axi), fy = floor_int(c64.ay, ayi);
+    Pre32& c32 = R.c32;
+    c32.gr = f32_of(c64.gr);
+    c32.gi = f32_of(c64.gi);
+    c32.axf = f32_of(c64.ax - fx);
+    c32.ayf = f32_of(c64.ay - fy);
+    c32.c1 = f32_of(c64.c1);
+    c32.c2 = f32_of(c64.c2);
+    c32.c3 = f32_of(c64.c3);
+    c32.c4 = f32_of(c64.c4);
+    c32.axi = axi;
+    c32.ayi = ayi;
+    c32.kx = 0x4B400000 - axi;
+    c32.ky = 0x4B400000 - ayi;
+  }
+  R.fl = fl;
 }
 
 // Combine pass entry idx (the render's prefix slots first, 4 nr of them:
 // last letter x, slot r0 + k; then the suffix slots).  prec: the kl_precision
 // of the render.  Fallback prefixes (KL_MIXED, KL_DF64) are appended to
-// fb_list as (group << 32) | slot.
+// fb_list as (group << 32) | slot.  filter: also the filter constants of the
+// prefixes on the FP64 or double-float map.
 __device__ void combine_entry(const View& V, const Plan& L, double ptol, int prec,
                               uint32_t idx, const Tables& T, uint32_t group,
                               unsigned long long* __restrict__ fb_list,
-                              uint32_t* __restrict__ fb_count) {
-  const bool mixed = prec == KL_MIXED, df = prec == KL_DF64;
+                              uint32_t* __restrict__ fb_count, bool filter) {
+  const bool df = prec == KL_DF64;
   const uint32_t nP = 4u * L.nr;
   if (idx >= nP) {
     const uint32_t slot = idx - nP;
@@ -497,71 +680,26 @@ __device__ void combine_entry(const View& V, const Plan& L, double ptol, int pre
   const int x = (int)(idx / L.nr);
   const uint32_t r = L.r0 + idx % L.nr;
   const uint32_t slot = (uint32_t)x * L.np + r;
-  const PartM& TL = T.Lt[(uint32_t)x * L.p3_q1 + r / L.p3_pq];
-  const M2 P = L.p > L.q ? mmul(T.Ht[(uint32_t)TL.edge * L.p3_pq + r % L.p3_pq], TL.m) : TL.m;
-  const dc det = mdet(P);
-  const dc tr = cadd(P.p, P.s);
-  const double scale = fmax(fmax(cabs1(P.p), cabs1(P.q)), fmax(cabs1(P.r), cabs1(P.s)));
-  uint32_t fl = 0;
-  const dc tr2m4 = csub(cmul(tr, tr), {4.0 * det.re, 4.0 * det.im});
-  const double t2 = tr.re * tr.re + tr.im * tr.im;
-  const double lim2 = ptol * fmax(1.0, t2);
-  if (tr2m4.re * tr2m4.re + tr2m4.im * tr2m4.im < lim2 * lim2) fl |= kNearPar;
-  Pre64 c64;
-  Pre32 c32;
-  if (!(cabs1(P.r) > 1e-12 * scale)) {
-    fl |= kDirect;
-    c64 = {P.p.re, P.p.im, P.q.re, P.q.im, P.r.re, P.r.im, P.s.re, P.s.im};
-    c32 = {};
-  } else {
-    const dc inv10 = crcp(P.r);
-    const dc alpha = cmul(P.p, inv10);
-    const dc gamma = cmul(P.s, inv10);
-    const dc mbeta = cmul(det, cmul(inv10, inv10));  // -beta
-    const double ax = (alpha.re - V.x0) * V.sx;
-    const double ay = (V.y1 - alpha.im) * V.sy;
-    const double c1 = -V.sx * mbeta.re, c2 = -V.sx * mbeta.im;
-    const double c3 = V.sy * mbeta.im, c4 = -V.sy * mbeta.re;
-    c64 = {gamma.re, gamma.im, ax, ay, c1, c2, c3, c4};
-    const double lim = 1048576.0;  // 2^20
-    if (!(fabs(ax) < lim && fabs(ay) < lim && fabs(gamma.re) < 1e15 && fabs(gamma.im) < 1e15))
-      fl |= kWide;
-    const double axi = floor(fmax(fmin(ax, lim), -lim));
-    const double ayi = floor(fmax(fmin(ay, lim), -lim));
-    c32.gr = (float)gamma.re;
-    c32.gi = (float)gamma.im;
-    c32.axf = (float)(ax - axi);
-    c32.ayf = (float)(ay - ayi);
-    c32.c1 = (float)c1;
-    c32.c2 = (float)c2;
-    c32.c3 = (float)c3;
-    c32.c4 = (float)c4;
-    c32.axi = (int)axi;
-    c32.ayi = (int)ayi;
-    c32.kx = 0x4B400000 - (int)axi;
-    c32.ky = 0x4B400000 - (int)ayi;
-  }
-  if (df) {
-    // the double-float constants; a constant (nonzero) outside [1e-30, 1e30]
-    // would leave the float range in the per-word products
-    PreDF cd;
-    const double cv[8] = {c64.gr, c64.gi, c64.ax, c64.ay, c64.c1, c64.c2, c64.c3, c64.c4};
-    for (int q = 0; q < 8; ++q) {
-      split_df(cv[q], cd.h[q], cd.l[q]);
-      const double a = fabs(cv[q]);
-      if (!(a < 1e30) || (a != 0.0 && a < 1e-30)) fl |= kDfRange;
-    }
-    if (!(fl & kDirect)) T.predf[slot] = cd;
-  }
-  if ((mixed && (fl & (kDirect | kNearPar | kWide))) ||
-      (df && (fl & (kDirect | kWide | kDfRange)))) {
-    fl |= kFallback;
+  PrefixRec R;
+  prefix_rec(V, L, ptol, prec, T, x, r, R);
+  if (R.fl & kFallback) {
     const uint32_t k = atomicAdd(fb_count, 1u);
     fb_list[k] = ((unsigned long long)group << 32) | slot;
   }
-  T.pre64[slot] = c64;
-  T.pre32[slot] = c32;
-  T.flags[slot] = fl;
+  T.pre64[slot] = R.c64;
+  if (df && !(R.fl & kDirect)) T.predf[slot] = R.cd;
+  // prefixes on the FP32 map need its record, the others their filter
+  // constants in its place (kl_filter.cuh)
+  if (R.fl & kOnFp32) {
+    T.pre32[slot] = R.c32;
+  } else if (filter) {
+    PreF cf;
+    if (!(R.fl & kDirect) && filter_consts(V, R.c64, cf))
+      *filter_slot(T, slot) = cf;
+    else
+      R.fl |= kNoFilter;
+  }
+  T.flags[slot] = R.fl;
 }
 
 // ---------------------------------------------------------------------------
@@ -606,10 +744,13 @@ struct UnitTally {
 };
 
 // Warp-sum the four counters and add them once per warp (all lanes must call).
-__device__ __forceinline__ void publish_counts(uint32_t in_window, uint32_t words,
-                                               uint32_t fp64_words, uint32_t atomics,
+__device__ __forceinline__ void publish_counts(uint32_t in_window, unsigned long long words,
+                                               unsigned long long fp64_words, uint32_t atomics,
                                                unsigned long long* counters) {
-  unsigned long long a = in_window, b = words - in_window, c = fp64_words, e = atomics;
+  // a lane may count words in the window that another lane counts as words: the
+  // differences are taken modulo 2^64 and only their sum is meant
+  unsigned long long a = in_window, b = words - in_window, c = fp64_words,
+                     e = atomics;
   for (int o = 16; o > 0; o >>= 1) {
     a += __shfl_down_sync(0xFFFFFFFFu, a, o);
     b += __shfl_down_sync(0xFFFFFFFFu, b, o);
@@ -742,23 +883,6 @@ __device__ __forceinline__ void words64(const Pre64& k, bool direct, const doubl
   }
   t.flush(img);
   if (BBOX) box_merge(*B, slot, c0, c1, r0, r1);
-}
-
-// One FP64 item of a plain render: words of this thread's prefix on one chunk.
-template <int BT>
-__device__ __forceinline__ void fp64_item(uint32_t item, const Work& Wk, const Plan& L,
-                                          const View& V, const Tables& T, Tally& t,
-                                          uint32_t& words, uint32_t* __restrict__ img) {
-  int x, u;
-  uint32_t pb, c;
-  item_of(item, Wk, x, u, pb, c);
-  const uint32_t k = pb * BT + threadIdx.x;
-  if (k >= L.nr) return;
-  const uint32_t slot = (uint32_t)x * L.np + L.r0 + k;
-  const uint32_t j0 = c * Wk.chunk, j1 = min(L.ns, j0 + Wk.chunk);
-  words64(T.pre64[slot], T.flags[slot] & kDirect, T.suf64 + (size_t)u * L.ns, j0, j1, V, t,
-          img);
-  words += j1 - j0;
 }
 
 // Mixed-mode FP64 fallback unit (kept out of line so that its registers do
@@ -904,5 +1028,6 @@ __device__ __forceinline__ void mixed_item(uint32_t item, const Work& Wk, const 
 
 // The double-float arithmetic, the culled renders and the host helpers.
 #include "kl_df.cuh"
+#include "kl_filter.cuh"
 #include "kl_cull.cuh"
 #include "kl_plan.cuh"

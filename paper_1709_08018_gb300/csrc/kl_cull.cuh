@@ -201,14 +201,17 @@ __device__ __forceinline__ void cull_disk(const Plan& L, const Tables& T, uint32
 // the FP32 one where that is finite and nonzero, since the FP32 entries are
 // the FP64 ones rounded).
 __device__ __forceinline__ void cull_norm(const Tables& T, uint32_t slot) {
-  const Pre32 k = T.pre32[slot];
-  const float n32 = opnorm32(k.c1, k.c2, k.c3, k.c4);
+  const bool on_fp32 = T.flags[slot] & kOnFp32;
+  const Pre32* k = T.pre32 + slot;
+  const Pre64* c64 = T.pre64 + slot;
+  const float n32 = on_fp32 ? opnorm32(k->c1, k->c2, k->c3, k->c4)
+                            : opnorm32((float)c64->c1, (float)c64->c2, (float)c64->c3,
+                                       (float)c64->c4);
   T.nrm32[slot] = n32;
   if (isfinite(n32) && n32 > 0.0f) {
     T.nrm64[slot] = (double)n32 * (1.0 + 0x1p-20);
-  } else {
-    const Pre64 c = T.pre64[slot];
-    T.nrm64[slot] = opnorm64(c.c1, c.c2, c.c3, c.c4);
+  } else if (!on_fp32) {
+    T.nrm64[slot] = opnorm64(c64->c1, c64->c2, c64->c3, c64->c4);
   }
 }
 

@@ -157,71 +157,6 @@ __device__ __forceinline__ void floor_keys(const DD& u, uint32_t& ka, uint32_t& 
   kb = (uint32_t)(t >> 32) - (db ? 1u : 0u);
 }
 
-// One run of n words ending in the pixel of keys (cu, cv) (absolute pixel
-// keys: col = cu - 0x4B400000).
-__device__ __forceinline__ void flush_key(uint32_t cu, uint32_t cv, uint32_t n, const View& V,
-                                          Tally& t, uint32_t* __restrict__ img) {
-  const uint32_t col = cu - 0x4B400000u, row = cv - 0x4B400000u;
-  if (n && col < V.W && row < V.H) {
-    atomicAdd(img + row * V.W + col, n);
-    ++t.atomics;
-    t.in_window += n;
-  }
-}
-
-// Double-float words of prefix slot `slot` on suffix point pairs [k0, k1) of
-// first letter u, with the run-length splat of mixed_slot_words on pixel keys.
-__device__ __forceinline__ void df64_slot_words(uint32_t slot, int u, uint32_t k0, uint32_t k1,
-                                                const Plan& L, const View& V, const Tables& T,
-                                                Tally& t, uint32_t& words,
-                                                uint32_t* __restrict__ img) {
-  const DfConst K = df_const(T.predf[slot]);
-  const float4* src = T.sufdf + 2ull * (size_t)u * L.npairs;
-  t.flush(img);
-  t.cur = -1;
-  uint32_t cu = 0, cv = 0, run = 0;  // keys (0, 0): no in-window pixel
-  uint32_t e_run = k0;
-  for (uint32_t e = k0; e < k1; ++e) {
-    const float4 a = __ldg(src + 2 * e), b = __ldg(src + 2 * e + 1);
-    const DD vr = {pk(a.x, a.y), pk(a.z, a.w)}, vi = {pk(b.x, b.y), pk(b.z, b.w)};
-    DD U, Vv;
-    uv_df2(K, vr, vi, U, Vv);
-    uint32_t ua, ub, va, vb;
-    floor_keys(U, ua, ub);
-    floor_keys(Vv, va, vb);
-    if (!((ua == cu) & (ub == cu) & (va == cv) & (vb == cv))) {
-      const bool a_in = (ua == cu) & (va == cv);
-      const bool ab = (ua == ub) & (va == vb);
-      run += 2u * (e - e_run) + (a_in ? 1u : 0u);
-      e_run = e + 1;
-      flush_key(cu, cv, run, V, t, img);
-      if (!a_in && !ab) flush_key(ua, va, 1u, V, t, img);  // word a on its own
-      run = (!a_in && ab) ? 2u : 1u;
-      cu = ub;
-      cv = vb;
-    }
-  }
-  run += 2u * (k1 - e_run);
-  flush_key(cu, cv, run, V, t, img);
-  words += min(2u * k1, L.ns) - 2u * k0;
-}
-
-// One double-float item: this thread's prefix on one chunk of suffix pairs.
-template <int BT>
-__device__ __forceinline__ void df64_item(uint32_t item, const Work& Wk, const Plan& L,
-                                          const View& V, const Tables& T, Tally& t,
-                                          uint32_t& words, uint32_t* __restrict__ img) {
-  int x, u;
-  uint32_t pb, c;
-  item_of(item, Wk, x, u, pb, c);
-  const uint32_t k = pb * BT + (threadIdx.x % BT);
-  if (k >= L.nr) return;
-  const uint32_t slot = (uint32_t)x * L.np + L.r0 + k;
-  if (T.flags[slot] & kFallback) return;
-  const uint32_t k0 = c * Wk.chunk, k1 = min(L.npairs, k0 + Wk.chunk);
-  df64_slot_words(slot, u, k0, k1, L, V, T, t, words, img);
-}
-
 // ---------------------------------------------------------------------------
 // scalar double-floats: one value per thread (the level-of-detail expansion,
 // where each lane holds its own node matrix).  The same arithmetic as the

@@ -194,6 +194,8 @@ inline View make_view(const kl_params* p) {
   memcpy(&bh, &h, sizeof bh);
   V.hiW = (uint32_t)(bw >> 32);
   V.hiH = (uint32_t)(bh >> 32);
+  V.kappa = (float)(V.sy / V.sx);
+  V.ik = (float)(V.sx / V.sy);
   return V;
 }
 

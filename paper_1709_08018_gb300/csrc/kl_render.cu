@@ -46,35 +46,19 @@ __global__ void parts_kernel(Group G, Plan L, int renorm, Tables T, Clear C,
 
 // Entries [first, combine_count): first = 4 nr (the prefixes skipped) when
 // the prefix tables are already in place.
-__global__ void combine_kernel(View V, Plan L, double ptol, int prec, Tables T, uint32_t first) {
+__global__ void combine_kernel(View V, Plan L, double ptol, int prec, Tables T, uint32_t first,
+                               int filter) {
   pdl_trigger();
   pdl_wait();
   const uint32_t total = combine_count(L);
   for (uint32_t idx = first + blockIdx.x * blockDim.x + threadIdx.x; idx < total;
        idx += gridDim.x * blockDim.x)
-    combine_entry(V, L, ptol, prec, idx, T, 0u, T.fb, T.fbcount);
+    combine_entry(V, L, ptol, prec, idx, T, 0u, T.fb, T.fbcount, filter != 0);
 }
 
 // ---------------------------------------------------------------------------
 // render kernels: persistent blocks drain a device work queue (one atomic per
 // item) of items of equal cost.
-
-// FP64: per item each thread evaluates its prefix on `chunk` consecutive
-// suffix points, read with a warp-uniform address (a broadcast from L1).
-template <int BT>
-__global__ void __launch_bounds__(BT) render64_kernel(Tables T, Plan L, View V, Work Wk,
-                                                      uint32_t* __restrict__ img,
-                                                      unsigned long long* counters) {
-  pdl_wait();
-  Tally t;
-  uint32_t words = 0;
-  for (;;) {
-    const uint32_t item = next_item(T.fbcount + 1);
-    if (item >= Wk.n_items) break;
-    fp64_item<BT>(item, Wk, L, V, T, t, words, img);
-  }
-  publish_counts(t.in_window, words, 0, t.atomics, counters);
-}
 
 // Mixed: the queue holds first the FP64 fallback items (32 units each: the
 // near-parabolic, direct-form and far prefixes), then the FP32 items (32
@@ -117,47 +101,24 @@ __global__ void __launch_bounds__(BT, 1280 / BT) render_mixed_kernel(
   publish_counts(t.in_window, words, fp64_words, t.atomics, counters);
 }
 
-// Double-float (KL_DF64): the queue holds first the FP64 fallback items (the
-// direct-form, far and out-of-float-range prefixes), then the double-float
-// items (32 prefixes x one chunk of suffix pairs), drawn per warp like the
-// mixed render's.  The per-word map is 117 FP32 operations in dependent
-// double-float chains, so the FMA pipe and the chains' latency, not issue,
-// bound the loop.  72 registers (7 blocks of 128 threads per SM): 2% faster
-// than at 82 registers (5 blocks) and than at 64 (8 blocks, spilling in the
-// loop); at 72 a few values are spilled per work item, not per word (local
-// loads are 0.01% of the instructions).
-template <int BT>
-__global__ void __launch_bounds__(BT, 896 / BT) render_df64_kernel(
+// FP64 and double-float words (the loop and its bound: kl_filter.cuh).
+// Each warp draws its own items, so warps never wait for one another.
+template <int BT, int PREC>
+__global__ void __launch_bounds__(BT, 1024 / BT) render_words_kernel(
     Tables T, Plan L, View V, Work Wk, uint32_t* __restrict__ img,
     unsigned long long* counters) {
+  __shared__ WarpQueue s_queue[BT / 32];
+  __shared__ ExactCtx C;
+  if (threadIdx.x == 0) C = {T, V, L.ns, L.npairs, img};
+  __syncthreads();
   pdl_wait();
-  const uint32_t chunks = (L.ns + kFbChunk - 1) / kFbChunk;
-  const uint32_t fb_units = 3u * chunks * (*T.fbcount);
-  const uint32_t n64 = (fb_units + 31) / 32;
-  const uint32_t total = n64 + Wk.n_items;
-  const uint32_t lane = threadIdx.x & 31;
-  Tally t;
-  uint32_t words = 0, fp64_words = 0;
+  WordWarp<PREC> w(&C, &s_queue[threadIdx.x >> 5]);
   for (;;) {
     const uint32_t item = next_item_warp(T.fbcount + 1);
-    if (item >= total) break;
-    if (item < n64) {
-      const uint32_t unit = item * 32 + lane;
-      if (unit < fb_units) {
-        const uint32_t e = unit / (3u * chunks), rem = unit % (3u * chunks);
-        const uint32_t slot = (uint32_t)(T.fb[e] & 0xFFFFFFFFull);
-        const UnitTally r = fallback_unit(T.pre64, T.flags, T.suf64, slot, rem / chunks,
-                                          rem % chunks, L.np, L.ns, V, img);
-        words += r.words;
-        fp64_words += r.words;
-        t.in_window += r.in_window;
-        t.atomics += r.atomics;
-      }
-      continue;
-    }
-    df64_item<32>(item - n64, Wk, L, V, T, t, words, img);
+    if (item >= Wk.n_items) break;
+    word_item(w, item, Wk, L, V, T, img);
   }
-  publish_counts(t.in_window, words, fp64_words, t.atomics, counters);
+  w.finish(counters);
 }
 
 // ---------------------------------------------------------------------------
@@ -357,7 +318,7 @@ int prof_mark(cudaEvent_t e, cudaStream_t s) {
 // fallback prefixes) are taken as they are and only the suffix side is built.
 int build_tables(const kl_params* p, const Plan& L, const View& V, const Group& G,
                  const Tables& T, cudaStream_t st, const Clear& C = Clear{},
-                 bool prefix_ready = false) {
+                 bool prefix_ready = false, bool filter = false) {
   const int prec = (int)p->precision;
   const uint32_t first_part = prefix_ready ? 4u * L.p3_q1 + (L.p > L.q ? 4u * L.p3_pq : 0u) : 0u;
   const uint32_t first_comb = prefix_ready ? 4u * L.nr : 0u;
@@ -375,7 +336,7 @@ int build_tables(const kl_params* p, const Plan& L, const View& V, const Group& 
   if (check_launch() != KL_OK) return KL_ECUDA;
   const uint32_t n = combine_count(L) - first_comb;
   return launch_dependent(combine_kernel, dim3(n > 0 ? (n + 127) / 128 : 1u), dim3(128), st, V,
-                          L, p->parabolic_tol, prec, T, first_comb);
+                          L, p->parabolic_tol, prec, T, first_comb, filter ? 1 : 0);
 }
 
 // Length k of a tiling render of *p: a limit-set render of the words of
@@ -426,6 +387,17 @@ int validate(const kl_params* p, size_t ws_bytes, void* ws, Plan* L) {
   return KL_OK;
 }
 
+using WordsKernel = void (*)(Tables, Plan, View, Work, uint32_t*, unsigned long long*);
+
+template <int BT>
+WordsKernel words_kernel(uint32_t precision) {
+  switch (precision) {
+    case KL_FP64: return render_words_kernel<BT, KL_FP64>;
+    case KL_DF64: return render_words_kernel<BT, KL_DF64>;
+    default: return render_mixed_kernel<BT>;
+  }
+}
+
 template <int BT>
 int launch_render(const kl_params* p, const Plan& L, const View& V, const Tables& T,
                   uint32_t* img, unsigned long long* cnt, cudaStream_t s, bool profile) {
@@ -450,35 +422,13 @@ int launch_render(const kl_params* p, const Plan& L, const View& V, const Tables
     if (st != KL_OK) return KL_ECUDA;
     return prof_mark(ev1, s);
   }
-  if (p->precision == KL_DF64) {
-    if (device_slots((const void*)render_df64_kernel<BT>, BT, &sms, &occ) != KL_OK)
-      return KL_ECUDA;
-    const Work Wk = make_work(L, 32, L.npairs, sms * occ * (BT / 32), p->chunk_pairs);
-    if (prof_mark(ev0, s) != KL_OK) return KL_ECUDA;
-    if (launch_dependent(render_df64_kernel<BT>, dim3(sms * occ), dim3(BT), s, T, L, V, Wk,
-                         img, cnt) != KL_OK)
-      return KL_ECUDA;
-    return prof_mark(ev1, s);
-  }
-  if (p->precision == KL_FP64) {
-    if (device_slots((const void*)render64_kernel<BT>, BT, &sms, &occ) != KL_OK) return KL_ECUDA;
-    // items of 64 suffix points by default: an FP64 item is slow (a 128-prefix block on
-    // 2,187 points takes milliseconds), so many small items keep the end of the queue
-    // even (0.7% faster than about 12 items per block at length 20)
-    const Work Wk = make_work(L, BT, L.ns, sms * occ, 2u * (p->chunk_pairs ? p->chunk_pairs : 32u));
-    if (prof_mark(ev0, s) != KL_OK) return KL_ECUDA;
-    if (launch_dependent(render64_kernel<BT>, dim3(sms * occ), dim3(BT), s, T, L, V, Wk, img,
-                         cnt) != KL_OK)
-      return KL_ECUDA;
-    return prof_mark(ev1, s);
-  }
-  if (device_slots((const void*)render_mixed_kernel<BT>, BT, &sms, &occ) != KL_OK)
-    return KL_ECUDA;
+  const void* k = (const void*)words_kernel<BT>(p->precision);
+  if (device_slots(k, BT, &sms, &occ) != KL_OK) return KL_ECUDA;
   // warp-sized items (32 prefixes), about 12 per resident warp
   const Work Wk = make_work(L, 32, L.npairs, sms * occ * (BT / 32), p->chunk_pairs);
   if (prof_mark(ev0, s) != KL_OK) return KL_ECUDA;
-  if (launch_dependent(render_mixed_kernel<BT>, dim3(sms * occ), dim3(BT), s, T, L, V, Wk, img,
-                       cnt) != KL_OK)
+  if (launch_dependent(words_kernel<BT>(p->precision), dim3(sms * occ), dim3(BT), s, T, L, V, Wk,
+                       img, cnt) != KL_OK)
     return KL_ECUDA;
   return prof_mark(ev1, s);
 }
@@ -566,7 +516,8 @@ int render_length(const kl_params* p, uint32_t* d_image, unsigned long long* cnt
   const Tables T = carve(L, d_workspace);
   Clear C{};
   if (!p->accumulate) C = {d_image, (size_t)p->width * p->height, cnt};
-  st = build_tables(p, L, V, G, T, s, C, prev && prefix_tables_shared(*prev, L, p));
+  const bool filter = p->precision != KL_MIXED && !p->cull;
+  st = build_tables(p, L, V, G, T, s, C, prev && prefix_tables_shared(*prev, L, p), filter);
   if (st != KL_OK) return st;
   switch (p->block_threads) {
     case 64: return launch_render<64>(p, L, V, T, d_image, cnt, s, profile);
