@@ -1,152 +1,255 @@
 // General presentations: the paper's own enumeration (Sec. "Implementation")
 // for any group given by an indexed Cayley table (Sec. "Cayley Multiplication
-// Tables").  Every index n of the unpruned m-ary tree of depth d is written as
-// d base-m digits plus one (symbols 1..m, w_1 most significant); the string
-// is kept when the table run over it, read right to left from state 0, never
-// reaches the crash state 0; a kept string is drawn at its word value (the
-// seed of w_d, then the maps of w_d, ..., w_1).
+// Tables").  Every index n of the unpruned m-ary tree of depth d is d base-m
+// digits plus one (symbols 1..m, w_1 most significant); the string is kept
+// when the table run over it, read right to left from state 0, never reaches
+// the crash state 0; a kept string is drawn at its word value (the seed of
+// w_d, then the maps of w_d, ..., w_1).
 //
-// GPU layout.  Each warp takes items of 32 x kPerLane consecutive indices;
-// lane l scans its own kPerLane indices with an odometer (the digits packed 4
-// bits each, the last digit, i.e. the first-applied letter, in the lowest
-// nibble), so no index is divided by m more than once per item.  The kept
-// strings are sparse (4 3^(d-1) of 4^d for the once-punctured torus), so the
-// warp compacts them: each round every lane tests one string, the kept ones
-// are appended to a per-warp queue in shared memory (ballot + prefix count),
-// and whenever the queue holds 32 words all lanes evaluate one each, with
-// every lane busy.  Word values are FP64; the splat is the run-length tally
-// of the other renders.
+// GPU layout.  A string is kept only if all its right ends are, and the value
+// of a right end is the point that the maps further left are applied to.  So
+// the kept strings are the leaves of a tree whose root side is w_d, and no
+// other string is ever looked at.  Each lane takes one kept right end of d - h
+// letters (a root, h <= 4), found by its rank: the numbers of kept strings of
+// every length from every state, counted on the host, say which symbol the
+// rank falls on.  It evaluates the root's point once and walks the root's
+// subtree of h more letters depth first, one map per node.  Scanning all m^d
+// strings, each kept one from its seed, took d FP64 maps per kept string and
+// was bound by the FP64 pipe (2 lanes per SM).  The walk takes (d - h) / 3^h
+// + 1/2 FP64 maps per kept string of the once-punctured torus: a leaf needs
+// only its pixel, so its own map is made in FP32 with an error bound, and in
+// FP64 (the same operations as for any node) when the bound does not settle
+// the pixel (a few leaves in 100; they wait in a queue until a warp has 32).  h = 4: roots enough to fill the
+// GPU from length 13 on; h = 3 leaves 1.4 times the FP64 maps (13 letters at
+// 2000 x 1500: 109 against 96 us, and 1624 us for the scan; the FP64 pipe's
+// share is 46 us).
 #include "kl_common.cuh"
 
 namespace {
 
-constexpr int kFsaThreads = 256;
-constexpr int kFsaWarps = kFsaThreads / 32;
-constexpr uint32_t kPerLane = 64;
+constexpr int kFsaThreads = 64;
 constexpr int kFsaMaxDepth = 32;
+constexpr int kFsaStates = KL_FSA_MAX_LETTERS + 1;
+constexpr int kFsaSubtree = 4;  // letters walked below a root, at most
 
 struct FsaDev {
   uint32_t m, d;
-  uint8_t table[(KL_FSA_MAX_LETTERS + 1) * (KL_FSA_MAX_LETTERS + 1)];
+  uint8_t table[kFsaStates * kFsaStates];  // row stride m + 1
   double g[KL_FSA_MAX_LETTERS * 8];
   double seed[KL_FSA_MAX_LETTERS * 2];
+  // ways[k][s]: strings of k symbols that run from state s without a crash
+  unsigned long long ways[kFsaMaxDepth + 1][kFsaStates];
 };
 
-// Packed digits: nibble k holds the symbol of w_{d-k} (k = 0: the first-
-// applied letter).  Two words of 16 nibbles cover d <= 32.
-struct Digits {
-  unsigned long long lo, hi;
+// One generator in FP32 with the 1-norms of its entries (the leaf test).
+struct FsaMap32 {
+  float v[8];           // p, q, r, s (re, im)
+  float np, nq, nr, ns;
 };
 
-__device__ __forceinline__ uint32_t nibble(const Digits& s, int k) {
-  return (uint32_t)((k < 16 ? s.lo >> (4 * k) : s.hi >> (4 * (k - 16))) & 15ull);
+// A block's shared tables.
+struct FsaShared {
+  uint32_t deg[kFsaStates];  // symbols that do not crash, per state
+  uint8_t sym[kFsaStates][KL_FSA_MAX_LETTERS], to[kFsaStates][KL_FSA_MAX_LETTERS];
+  double g[KL_FSA_MAX_LETTERS * 8];
+  double seed[KL_FSA_MAX_LETTERS * 2];
+  FsaMap32 f[KL_FSA_MAX_LETTERS];
+  unsigned long long ways[kFsaMaxDepth + 1][kFsaStates];
+};
+
+// One map in FP64 (a refined reciprocal instead of divisions), its multiply-adds
+// spelled out so that every string's value has the same bits wherever the
+// compiler inlines it.
+__device__ __forceinline__ double mul_sub(double a, double b, double c, double d) {
+  return __fma_rn(a, b, -__dmul_rn(c, d));
+}
+__device__ __forceinline__ double mul_add(double a, double b, double c, double d) {
+  return __fma_rn(a, b, __dmul_rn(c, d));
+}
+__device__ __forceinline__ dc fsa_map(const double* M, dc z) {
+  const dc num = {__dadd_rn(mul_sub(M[0], z.re, M[1], z.im), M[2]),
+                  __dadd_rn(mul_add(M[0], z.im, M[1], z.re), M[3])};
+  const dc den = {__dadd_rn(mul_sub(M[4], z.re, M[5], z.im), M[6]),
+                  __dadd_rn(mul_add(M[4], z.im, M[5], z.re), M[7])};
+  const double r = rcp64(mul_add(den.re, den.re, den.im, den.im));
+  return {__dmul_rn(mul_add(num.re, den.re, num.im, den.im), r),
+          __dmul_rn(mul_sub(num.im, den.re, num.re, den.im), r)};
 }
 
-// The string of index n (symbols = base-m digits plus one).
-__device__ Digits digits_of(unsigned long long n, uint32_t m, uint32_t d) {
-  Digits s{0ull, 0ull};
-  for (uint32_t k = 0; k < d; ++k) {
-    const unsigned long long sym = n % m + 1;
-    n /= m;
-    if (k < 16) s.lo |= sym << (4 * k);
-    else s.hi |= sym << (4 * (k - 16));
-  }
-  return s;
+// Pixel of map M of the point z (as FP32: zr, zi) where an FP32 evaluation
+// settles it, -1 for certainly outside the window, kUnsettled otherwise.
+// Error: numerator and denominator are sums of products of once-rounded
+// values, off by at most 6 eps A and 6 eps B per part (A = |p||z| + |q|, B =
+// |r||z| + |s| in 1-norms, eps = 2^-24); with 12 eps B < |den| / 4 the quotient w
+// is off by less than 12 eps (A + |w| B) / |den| plus 13 eps |w| for its own
+// roundings and the reciprocal root, and the pixel transform adds 5 eps of
+// |w| + |x0| (|y1|); the code takes 20 eps for the last two.
+constexpr int kUnsettled = -2;
+__device__ __forceinline__ int fsa_leaf32(const FsaMap32& M, float zr, float zi, const View& V,
+                                          float x0, float y1, float sx, float sy) {
+  const float* v = M.v;
+  const float nr = fmaf(v[0], zr, fmaf(-v[1], zi, v[2])), ni = fmaf(v[0], zi, fmaf(v[1], zr, v[3]));
+  const float dr = fmaf(v[4], zr, fmaf(-v[5], zi, v[6])), di = fmaf(v[4], zi, fmaf(v[5], zr, v[7]));
+  float rd;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rd) : "f"(fmaf(dr, dr, di * di)));
+  const float rc = rd * rd;
+  const float wr = fmaf(nr, dr, ni * di) * rc, wi = fmaf(ni, dr, -(nr * di)) * rc;
+  const float az = fabsf(zr) + fabsf(zi), aw = fabsf(wr) + fabsf(wi);
+  const float A = fmaf(M.np, az, M.nq), B = fmaf(M.nr, az, M.ns);
+  const float u = (wr - x0) * sx, w = (y1 - wi) * sy;
+  const float e = fmaf(12.0f * 0x1p-24f * rd, fmaf(aw, B, A), 20.0f * 0x1p-24f * aw);
+  const float eu = fmaf(5.0f * 0x1p-24f, fabsf(x0), e) * sx;
+  const float ew = fmaf(5.0f * 0x1p-24f, fabsf(y1), e) * sy;
+  if (!(12.0f * 0x1p-24f * B * rd < 0.25f && eu < 0.25f && ew < 0.25f)) return kUnsettled;
+  const float W = (float)V.W, H = (float)V.H;
+  if (u < -eu || u > W + eu || w < -ew || w > H + ew) return -1;
+  const int c0 = (int)floorf(u - eu), c1 = (int)floorf(u + eu);
+  const int r0 = (int)floorf(w - ew), r1 = (int)floorf(w + ew);
+  if (c0 != c1 || r0 != r1 || c0 < 0 || r0 < 0 || c0 >= (int)V.W || r0 >= (int)V.H)
+    return kUnsettled;
+  return r0 * (int)V.W + c0;
 }
 
-// n + 1: the lowest symbol steps up, symbols past m wrap to 1 and carry.
-__device__ __forceinline__ void step(Digits& s, uint32_t m, uint32_t d) {
-  for (uint32_t k = 0; k < d; ++k) {
-    const uint32_t v = nibble(s, (int)k);
-    const unsigned long long one = 1ull << (4 * (k & 15u));
-    unsigned long long& w = k < 16 ? s.lo : s.hi;
-    if (v < m) {
-      w += one;
-      return;
-    }
-    w -= (unsigned long long)(m - 1) * one;  // m -> 1, carry on
-  }
-}
+// A warp's queue of leaves that FP32 did not settle: the parent's point and
+// the generator.
+struct FsaQueue {
+  double zr[64], zi[64];
+  uint32_t x[64];
+};
 
-// Table run right to left from state 0; true if no crash.
-__device__ __forceinline__ bool kept(const Digits& s, const uint8_t* tab, uint32_t m,
-                                     uint32_t d) {
-  uint32_t state = 0;
-  for (uint32_t k = 0; k < d; ++k) {
-    state = tab[state * (m + 1) + nibble(s, (int)k)];
-    if (state == 0) return false;
-  }
-  return true;
-}
-
-// Word value, FP64: z = seed of w_d, then the maps of w_d, ..., w_1.
-__device__ __forceinline__ dc fsa_value(const Digits& s, const double* g, const double* seed,
-                                        uint32_t d) {
-  const uint32_t x0 = nibble(s, 0) - 1;
-  dc z = {seed[2 * x0], seed[2 * x0 + 1]};
-  for (uint32_t k = 0; k < d; ++k) {
-    const double* M = g + 8 * (nibble(s, (int)k) - 1);
-    const dc num = {M[0] * z.re - M[1] * z.im + M[2], M[0] * z.im + M[1] * z.re + M[3]};
-    const dc den = {M[4] * z.re - M[5] * z.im + M[6], M[4] * z.im + M[5] * z.re + M[7]};
-    const double r = rcp64(den.re * den.re + den.im * den.im);
-    z = {(num.re * den.re + num.im * den.im) * r, (num.im * den.re - num.re * den.im) * r};
-  }
-  return z;
-}
-
-__global__ void __launch_bounds__(kFsaThreads) fsa_render_kernel(
-    FsaDev F, View V, unsigned long long n_idx, unsigned long long n_items,
-    unsigned long long* queue, uint32_t* __restrict__ img, unsigned long long* counters) {
-  // (the evaluated words of one thread fit uint32: a thread evaluates at most
-  // one word per 32 scanned strings of its warp's items)
-  __shared__ uint8_t tab[(KL_FSA_MAX_LETTERS + 1) * (KL_FSA_MAX_LETTERS + 1)];
-  __shared__ double g[KL_FSA_MAX_LETTERS * 8];
-  __shared__ double seed[KL_FSA_MAX_LETTERS * 2];
-  __shared__ Digits wq[kFsaWarps][64];
-  for (int i = threadIdx.x; i < (int)((F.m + 1) * (F.m + 1)); i += blockDim.x) tab[i] = F.table[i];
-  for (int i = threadIdx.x; i < (int)(8 * F.m); i += blockDim.x) g[i] = F.g[i];
-  for (int i = threadIdx.x; i < (int)(2 * F.m); i += blockDim.x) seed[i] = F.seed[i];
-  __syncthreads();
-  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const unsigned lt = (1u << lane) - 1u;
-  Digits* q = wq[warp];
-  uint32_t qlen = 0;
+// What a walk carries along.  All lanes of a warp walk together (`on`: this
+// lane's node exists), over the largest number of symbols any state has.
+struct FsaWalk {
+  const FsaShared* S;
+  FsaQueue* Q;
+  View V;
+  float x0, y1, sx, sy;
+  uint32_t* img;
+  uint32_t most, len, words;
   Tally t;
-  uint32_t evaluated = 0;
-  auto drain = [&](uint32_t k) {  // evaluate queue entries [0, k) (k <= 32), one per lane
-    if (lane < k) {
-      const dc z = fsa_value(q[lane], g, seed, F.d);
-      t.add(pixel64((z.re - V.x0) * V.sx, (V.y1 - z.im) * V.sy, V), img);
-      ++evaluated;
-    }
-    __syncwarp();
-  };
-  for (;;) {
-    unsigned long long item = 0;
-    if (lane == 0) item = atomicAdd(queue, 1ull);
-    item = __shfl_sync(0xFFFFFFFFu, item, 0);
-    if (item >= n_items) break;
-    const unsigned long long first = item * 32ull * kPerLane + (unsigned long long)lane * kPerLane;
-    Digits s = digits_of(first < n_idx ? first : 0ull, F.m, F.d);
-    for (uint32_t r = 0; r < kPerLane; ++r) {
-      const bool ok = first + r < n_idx && kept(s, tab, F.m, F.d);
-      const unsigned b = __ballot_sync(0xFFFFFFFFu, ok);
-      if (ok) q[qlen + __popc(b & lt)] = s;
-      qlen += __popc(b);
-      __syncwarp();
-      if (qlen >= 32) {
-        drain(32);
-        qlen -= 32;
-        if (lane < qlen) q[lane] = q[32 + lane];
-        __syncwarp();
+};
+
+__device__ __forceinline__ void fsa_word(FsaWalk& w, dc z) {
+  w.t.add(pixel64((z.re - w.V.x0) * w.V.sx, (w.V.y1 - z.im) * w.V.sy, w.V), w.img);
+}
+// queue entries [len - n, len), one per lane
+__device__ __forceinline__ void fsa_drain(FsaWalk& w, uint32_t n) {
+  __syncwarp();
+  const uint32_t lane = threadIdx.x & 31, k = w.len - n + lane;
+  if (lane < n) fsa_word(w, fsa_map(w.S->g + 8 * w.Q->x[k], {w.Q->zr[k], w.Q->zi[k]}));
+  w.len -= n;
+  __syncwarp();
+}
+
+// The kept strings h letters further left of a right end with point z that
+// left the run in `state`.
+template <int h>
+__device__ __forceinline__ void fsa_walk(FsaWalk& w, bool on, uint32_t state, dc z) {
+  const FsaShared& S = *w.S;
+  if constexpr (h == 0) {
+    if (on) fsa_word(w, z);
+    w.words += on;
+  } else if constexpr (h == 1) {
+    const uint32_t n = on ? S.deg[state] : 0u;
+    const float zr = f32_of(z.re), zi = f32_of(z.im);
+    w.words += n;
+#pragma unroll 1
+    for (uint32_t k = 0; k < w.most; ++k) {
+      int pix = -1;
+      uint32_t x = 0;
+      if (k < n) {
+        x = S.sym[state][k];
+        pix = fsa_leaf32(S.f[x], zr, zi, w.V, w.x0, w.y1, w.sx, w.sy);
+        if (pix != kUnsettled) w.t.add(pix, w.img);
       }
-      step(s, F.m, F.d);
+      const unsigned b = __ballot_sync(0xFFFFFFFFu, pix == kUnsettled);
+      if (b) {
+        if (pix == kUnsettled) {
+          const uint32_t at = w.len + __popc(b & ((1u << (threadIdx.x & 31)) - 1u));
+          w.Q->zr[at] = z.re;
+          w.Q->zi[at] = z.im;
+          w.Q->x[at] = x;
+        }
+        w.len += __popc(b);
+        if (w.len >= 32) fsa_drain(w, 32);
+      }
+    }
+  } else {
+    const uint32_t n = on ? S.deg[state] : 0u;
+#pragma unroll 1
+    for (uint32_t k = 0; k < w.most; ++k) {
+      const bool child = k < n;
+      const uint32_t x = child ? S.sym[state][k] : 0u;
+      fsa_walk<h - 1>(w, child, child ? S.to[state][k] : 0u, fsa_map(S.g + 8 * x, z));
     }
   }
-  drain(qlen);
-  t.flush(img);
-  publish_counts(t.in_window, evaluated, evaluated, t.atomics, counters);
 }
+
+template <int h>
+__global__ void __launch_bounds__(kFsaThreads) fsa_render_kernel(
+    const __grid_constant__ FsaDev F, View V, uint32_t* __restrict__ img,
+    unsigned long long* counters) {
+  __shared__ FsaShared S;
+  __shared__ FsaQueue queues[kFsaThreads / 32];
+  const uint32_t m = F.m;
+  for (uint32_t i = threadIdx.x; i < 8u * m; i += kFsaThreads) S.g[i] = F.g[i];
+  for (uint32_t i = threadIdx.x; i < 2u * m; i += kFsaThreads) S.seed[i] = F.seed[i];
+  for (uint32_t i = threadIdx.x; i < 8u * m; i += kFsaThreads) S.f[i / 8].v[i % 8] = (float)F.g[i];
+  for (uint32_t i = threadIdx.x; i < (F.d + 1) * kFsaStates; i += kFsaThreads)
+    S.ways[i / kFsaStates][i % kFsaStates] = F.ways[i / kFsaStates][i % kFsaStates];
+  if (threadIdx.x <= m) {
+    const uint32_t s = threadIdx.x;
+    uint32_t n = 0;
+    for (uint32_t y = 1; y <= m; ++y) {
+      const uint32_t to = F.table[s * (m + 1) + y];
+      if (!to) continue;
+      S.sym[s][n] = (uint8_t)(y - 1);
+      S.to[s][n++] = (uint8_t)to;
+    }
+    S.deg[s] = n;
+  }
+  __syncthreads();
+  if (threadIdx.x < m) {
+    FsaMap32& f = S.f[threadIdx.x];
+    f.np = fabsf(f.v[0]) + fabsf(f.v[1]);
+    f.nq = fabsf(f.v[2]) + fabsf(f.v[3]);
+    f.nr = fabsf(f.v[4]) + fabsf(f.v[5]);
+    f.ns = fabsf(f.v[6]) + fabsf(f.v[7]);
+  }
+  __syncthreads();
+  FsaWalk w = {&S, &queues[threadIdx.x / 32], V, (float)V.x0, (float)V.y1, (float)V.sx,
+               (float)V.sy, img, 0u, 0u, 0u, Tally()};
+  for (uint32_t s = 1; s <= m; ++s) w.most = max(w.most, S.deg[s]);  // (0 only starts a run)
+  const uint32_t l = F.d - h;
+  const unsigned long long roots = F.ways[l][0];
+  for (unsigned long long first = blockIdx.x * (unsigned long long)kFsaThreads;
+       first < roots; first += (unsigned long long)gridDim.x * kFsaThreads) {
+    const bool on = first + threadIdx.x < roots;
+    // the root of that rank, innermost letter first
+    unsigned long long r = on ? first + threadIdx.x : 0ull;
+    uint32_t state = 0;
+    dc z = {0.0, 0.0};
+#pragma unroll 1
+    for (uint32_t k = 0; k < l; ++k) {
+      uint32_t i = 0;
+      for (;; ++i) {
+        const unsigned long long c = S.ways[l - 1 - k][S.to[state][i]];
+        if (r < c) break;
+        r -= c;
+      }
+      const uint32_t x = S.sym[state][i];
+      state = S.to[state][i];
+      if (k == 0) z = {S.seed[2 * x], S.seed[2 * x + 1]};
+      z = fsa_map(S.g + 8 * x, z);
+    }
+    fsa_walk<h>(w, on, state, z);
+  }
+  fsa_drain(w, w.len);
+  w.t.flush(img);
+  publish_counts(w.t.in_window, w.words, w.words, w.t.atomics, counters);
+}
+
+using FsaKernel = void (*)(FsaDev, View, uint32_t*, unsigned long long*);
 
 int fsa_check(const kl_fsa* f, uint32_t d, unsigned long long* n_idx) {
   if (!f || f->m < 1 || f->m > KL_FSA_MAX_LETTERS) return KL_EINVAL;
@@ -167,6 +270,23 @@ int fsa_check(const kl_fsa* f, uint32_t d, unsigned long long* n_idx) {
   return KL_OK;
 }
 
+// ways[k][s] of FsaDev for k <= depth.
+void fsa_ways(const kl_fsa* f, uint32_t depth,
+              unsigned long long (*ways)[kFsaStates]) {
+  const uint32_t m = f->m;
+  for (uint32_t s = 0; s <= m; ++s) ways[0][s] = 1;
+  // one more symbol in front: the sum over symbols of the non-crash targets' ways
+  for (uint32_t k = 0; k < depth; ++k)
+    for (uint32_t s = 0; s <= m; ++s) {
+      unsigned long long acc = 0;
+      for (uint32_t sym = 1; sym <= m; ++sym) {
+        const uint32_t to = f->table[s * kFsaStates + sym];
+        if (to != 0) acc += ways[k][to];
+      }
+      ways[k + 1][s] = acc;
+    }
+}
+
 }  // namespace
 
 extern "C" int kl_fsa_count(const kl_fsa* f, uint32_t depth, uint64_t* count) {
@@ -174,24 +294,9 @@ extern "C" int kl_fsa_count(const kl_fsa* f, uint32_t depth, uint64_t* count) {
   const int st = fsa_check(f, depth, &n_idx);
   if (st != KL_OK) return st;
   if (!count) return KL_EINVAL;
-  // ways[s] = strings of the remaining length that run from state s without a
-  // crash; one more symbol in front of the run: ways'(s) = sum over symbols
-  // of ways(table[s][symbol]) for non-crash targets.
-  const uint32_t m = f->m;
-  unsigned long long ways[KL_FSA_MAX_LETTERS + 1], next[KL_FSA_MAX_LETTERS + 1];
-  for (uint32_t s = 0; s <= m; ++s) ways[s] = 1;
-  for (uint32_t k = 0; k < depth; ++k) {
-    for (uint32_t s = 0; s <= m; ++s) {
-      unsigned long long acc = 0;
-      for (uint32_t sym = 1; sym <= m; ++sym) {
-        const uint32_t to = f->table[s * (KL_FSA_MAX_LETTERS + 1) + sym];
-        if (to != 0) acc += ways[to];
-      }
-      next[s] = acc;
-    }
-    for (uint32_t s = 0; s <= m; ++s) ways[s] = next[s];
-  }
-  *count = ways[0];
+  unsigned long long ways[kFsaMaxDepth + 1][kFsaStates];
+  fsa_ways(f, depth, ways);
+  *count = ways[depth][0];
   return KL_OK;
 }
 
@@ -221,14 +326,18 @@ extern "C" int kl_render_fsa(const kl_fsa* f, const kl_params* p, uint32_t* d_im
     F.table[i] = f->table[(i / (F.m + 1)) * (KL_FSA_MAX_LETTERS + 1) + i % (F.m + 1)];
   for (uint32_t k = 0; k < 8 * F.m; ++k) F.g[k] = f->gens[k];
   for (uint32_t k = 0; k < 2 * F.m; ++k) F.seed[k] = f->seeds[k];
+  fsa_ways(f, F.d, F.ways);
+  const uint32_t h = F.d - 1 < (uint32_t)kFsaSubtree ? F.d - 1 : (uint32_t)kFsaSubtree;
+  const FsaKernel kernels[kFsaSubtree + 1] = {fsa_render_kernel<0>, fsa_render_kernel<1>,
+                                              fsa_render_kernel<2>, fsa_render_kernel<3>,
+                                              fsa_render_kernel<4>};
   int sms = 0, occ = 0;
-  if (device_slots((const void*)fsa_render_kernel, kFsaThreads, &sms, &occ) != KL_OK)
-    return KL_ECUDA;
-  const unsigned long long per_item = 32ull * kPerLane;
-  const unsigned long long n_items = (n_idx + per_item - 1) / per_item;
-  unsigned long long* queue = (unsigned long long*)d_workspace;  // the item queue head
-  if (cudaMemsetAsync(queue, 0, sizeof(unsigned long long), s) != cudaSuccess) return KL_ECUDA;
-  fsa_render_kernel<<<sms * occ, kFsaThreads, 0, s>>>(F, make_view(p), n_idx, n_items, queue,
-                                                      d_image, cnt);
+  if (device_slots((const void*)kernels[h], kFsaThreads, &sms, &occ) != KL_OK) return KL_ECUDA;
+  const unsigned long long roots = F.ways[F.d - h][0];
+  const unsigned long long blocks = (roots + kFsaThreads - 1) / kFsaThreads;
+  const unsigned long long most = (unsigned long long)sms * occ;
+  if (blocks == 0) return KL_OK;
+  kernels[h]<<<(unsigned)(blocks < most ? blocks : most), kFsaThreads, 0, s>>>(F, make_view(p),
+                                                                            d_image, cnt);
   return check_launch();
 }
