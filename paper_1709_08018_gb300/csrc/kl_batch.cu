@@ -54,7 +54,8 @@ __global__ void batch_parts_kernel(const GroupDesc* __restrict__ D,
 
 __global__ void batch_combine_kernel(const GroupDesc* __restrict__ D,
                                      const uint32_t* __restrict__ bases, uint32_t n,
-                                     uint32_t total, int mixed, int filter, unsigned long long* fb,
+                                     uint32_t total, int mixed, WordTables what,
+                                     unsigned long long* fb,
                                      uint32_t* fb_count) {
   for (uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total;
        idx += gridDim.x * blockDim.x) {
@@ -62,7 +63,7 @@ __global__ void batch_combine_kernel(const GroupDesc* __restrict__ D,
     const Plan L = D[g].L;
     const View V = D[g].V;
     const Tables T = D[g].T;
-    combine_entry(V, L, D[g].ptol, mixed, idx - bases[g], T, g, fb, fb_count, filter != 0);
+    combine_entry(V, L, D[g].ptol, mixed, idx - bases[g], T, g, fb, fb_count, what);
   }
 }
 
@@ -348,7 +349,8 @@ int enqueue(kl_batch* b, uint32_t* images, uint64_t* counters, void* ws, cudaStr
   if (check_launch() != KL_OK) return KL_ECUDA;
   const uint32_t gc = (b->n_comb + 127) / 128;
   batch_combine_kernel<<<gc < 1048576u ? gc : 1048576u, 128, 0, s>>>(
-      D, bases + (n + 1), n, b->n_comb, b->mixed, !b->mixed && !b->cull, fb, cnt2);
+      D, bases + (n + 1), n, b->n_comb, b->mixed,
+      b->cull ? kCullTables : b->mixed ? kPlainTables : kFilterTables, fb, cnt2);
   if (check_launch() != KL_OK) return KL_ECUDA;
   if (b->cull) {
     const uint32_t gd = (b->n_disk + 3) / 4;  // four warps per block

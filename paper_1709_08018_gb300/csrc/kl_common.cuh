@@ -46,6 +46,15 @@ constexpr uint32_t kFallback = 8u;   // KL_MIXED, KL_DF64: words of this prefix 
 constexpr uint32_t kDfRange = 16u;   // a pole-form constant outside the double-float range
 constexpr uint32_t kNoFilter = 32u;  // no filter constants: words take the exact map (kl_filter.cuh)
 constexpr uint32_t kOnFp32 = 64u;    // KL_MIXED: words on the FP32 map (its record is pre32's)
+constexpr uint32_t kNear32 = 128u;   // words on the FP64 map, with an FP32 record for the certified
+                                     // tests of a culled render
+
+// What the words of a render read beside the FP64 records (combine_entry).
+enum WordTables : int {
+  kPlainTables,   // FP32 records of the prefixes on the FP32 map
+  kFilterTables,  // filter constants (kl_filter.cuh)
+  kCullTables     // FP32 records of all prefixes in range (kl_cull.cuh)
+};
 
 // FP64 fallback work unit: a chunk of this many suffix points.
 constexpr uint32_t kFbChunk = 64;
@@ -255,13 +264,19 @@ __device__ __forceinline__ void uv_pole64(const Pre64& c, double vr, double vi, 
 }
 
 // Direct form for prefixes whose P10 vanishes: z = (P00 v + P01)/(P10 v + P11).
+// Its multiply-adds are spelled out so that a word's value has the same bits in
+// every kernel that evaluates it.
 __device__ __forceinline__ void uv_direct64(const Pre64& c, double vr, double vi,
                                             const View& V, double& u, double& v) {
-  dc P00 = {c.gr, c.gi}, P01 = {c.ax, c.ay}, P10 = {c.c1, c.c2}, P11 = {c.c3, c.c4};
-  dc z = {vr, vi};
-  dc w = cdiv(cadd(cmul(P00, z), P01), cadd(cmul(P10, z), P11));
-  u = (w.re - V.x0) * V.sx;
-  v = (V.y1 - w.im) * V.sy;
+  const double nr = __dadd_rn(__fma_rn(c.gr, vr, -__dmul_rn(c.gi, vi)), c.ax);
+  const double ni = __dadd_rn(__fma_rn(c.gr, vi, __dmul_rn(c.gi, vr)), c.ay);
+  const double mr = __dadd_rn(__fma_rn(c.c1, vr, -__dmul_rn(c.c2, vi)), c.c3);
+  const double mi = __dadd_rn(__fma_rn(c.c1, vi, __dmul_rn(c.c2, vr)), c.c4);
+  const double den = __fma_rn(mr, mr, __dmul_rn(mi, mi));
+  const double zr = __ddiv_rn(__fma_rn(nr, mr, __dmul_rn(ni, mi)), den);
+  const double zi = __ddiv_rn(__fma_rn(ni, mr, -__dmul_rn(nr, mi)), den);
+  u = __dmul_rn(__dsub_rn(zr, V.x0), V.sx);
+  v = __dmul_rn(__dsub_rn(V.y1, zi), V.sy);
 }
 
 // Scalar form of the mixed per-word map (the evaluation kernel); the render
@@ -524,16 +539,35 @@ __device__ __forceinline__ bool filter_consts(const View& V, const Pre64& c, Pre
          fabsf(f.ayf) < 1e30f && V.ik > 1e-6f && V.ik < 1e6f;
 }
 
-// The filter constants of a slot lie in its FP32 record, which prefixes on the
-// FP64 or double-float map do not read.
+// The filter constants of a slot lie in its FP32 record's place: a filtered
+// render forms that record from the FP64 one for the few words that need it.
 __device__ __forceinline__ PreF* filter_slot(const Tables& T, uint32_t slot) {
   return reinterpret_cast<PreF*>(T.pre32 + slot);
+}
+
+// The FP32 record of a prefix on the FP32 map (kOnFp32).
+__device__ __forceinline__ Pre32 pre32_of(const Pre64& c64) {
+  Pre32 c32;
+  int axi, ayi;
+  const double fx = floor_int(c64.ax, axi), fy = floor_int(c64.ay, ayi);
+  c32.gr = f32_of(c64.gr);
+  c32.gi = f32_of(c64.gi);
+  c32.axf = f32_of(c64.ax - fx);
+  c32.ayf = f32_of(c64.ay - fy);
+  c32.c1 = f32_of(c64.c1);
+  c32.c2 = f32_of(c64.c2);
+  c32.c3 = f32_of(c64.c3);
+  c32.c4 = f32_of(c64.c4);
+  c32.axi = axi;
+  c32.ayi = ayi;
+  c32.kx = 0x4B400000 - axi;
+  c32.ky = 0x4B400000 - ayi;
+  return c32;
 }
 
 // Everything the words of one prefix need.
 struct PrefixRec {
   Pre64 c64;
-  Pre32 c32;  // KL_MIXED, not kFallback
   PreDF cd;   // KL_DF64, not kDirect
   uint32_t fl;
 };
@@ -604,77 +638,66 @@ __device__ __forceinline__ void prefix_rec(const View& V, const Plan& L, double 
   if ((mixed && (fl & (kDirect | kNearPar | kWide))) ||
       (df && (fl & (kDirect | kWide | kDfRange))))
     fl |= kFallback;
-  if (mixed && !(fl & kFallback)) {
-    fl |= kOnFp32;
-    int axi, ayi;
-    const double fx = floor_int(c64.ax, axi), fy = floor_int(c64.ay, ayi);
-    Pre32& c32 = R.c32;
-    c32.gr = f32_of(c64.gr);
-    c32.gi = f32_of(c64.gi);
-    c32.axf = f32_of(c64.ax - fx);
-    c32.ayf = f32_of(c64.ay - fy);
-    c32.c1 = f32_of(c64.c1);
-    c32.c2 = f32_of(c64.c2);
-    c32.c3 = f32_of(c64.c3);
-    c32.c4 = f32_of(c64.c4);
-    c32.axi = axi;
-    c32.ayi = ayi;
-    c32.kx = 0x4B400000 - axi;
-    c32.ky = 0x4B400000 - ayi;
-  }
+  if (mixed && !(fl & kFallback)) fl |= kOnFp32;
   R.fl = fl;
+}
+
+// Suffix slot `slot` of the combine pass: the suffix point in the formats that
+// the words of precision prec read.
+__device__ __forceinline__ void suffix_entry(const Plan& L, int prec, uint32_t slot,
+                                             const Tables& T) {
+  const bool df = prec == KL_DF64;
+  double2 v;
+  if (L.so == 0) {
+    v = T.Sit[slot];
+  } else {
+    const int u = (int)(slot / L.ns);
+    const uint32_t j = slot % L.ns;
+    const uint32_t j_so = j / L.p3_si, rem = j % L.p3_si;
+    const PartM& S = T.Sot[(uint32_t)u * L.p3_so1 + j_so];
+    const int z = allowed_letter((int)(rem / L.p3_si1), (S.edge + 2) & 3);
+    const double2 t = T.Sit[(uint32_t)z * L.p3_si1 + rem % L.p3_si1];
+    const dc r = mobius(S.m, {t.x, t.y});
+    v = make_double2(r.re, r.im);
+  }
+  T.suf64[slot] = v;
+  // pair-interleaved FP32 table: per first letter u, entry k holds
+  // (re v_2k, re v_2k+1, im v_2k, im v_2k+1); an odd count is padded with NaN
+  const uint32_t u = slot / L.ns, j = slot % L.ns;
+  float* e = (float*)T.suf32p + 4ull * ((uint64_t)u * L.npairs + j / 2u);
+  e[j & 1u] = (float)v.x;
+  e[2 + (j & 1u)] = (float)v.y;
+  if (j + 1u == L.ns && (L.ns & 1u)) {
+    e[1] = __int_as_float(0x7FC00000);
+    e[3] = __int_as_float(0x7FC00000);
+  }
+  if (df) {
+    // pair-interleaved double-float table, padded with NaN like the FP32 one
+    float* q = (float*)T.sufdf + 8ull * ((uint64_t)u * L.npairs + j / 2u);
+    float rh, rl, ih, il;
+    split_df(v.x, rh, rl);
+    split_df(v.y, ih, il);
+    q[j & 1u] = rh;
+    q[2 + (j & 1u)] = rl;
+    q[4 + (j & 1u)] = ih;
+    q[6 + (j & 1u)] = il;
+    if (j + 1u == L.ns && (L.ns & 1u))
+      for (int c = 1; c < 8; c += 2) q[c] = __int_as_float(0x7FC00000);
+  }
 }
 
 // Combine pass entry idx (the render's prefix slots first, 4 nr of them:
 // last letter x, slot r0 + k; then the suffix slots).  prec: the kl_precision
-// of the render.  Fallback prefixes (KL_MIXED, KL_DF64) are appended to
-// fb_list as (group << 32) | slot.  filter: also the filter constants of the
-// prefixes on the FP64 or double-float map.
+// of the render.  kFilterTables: the filter constants lie in the FP32 record's
+// place; kPlainTables: fallback prefixes (KL_MIXED) are appended to fb_list as
+// (group << 32) | slot.
 __device__ void combine_entry(const View& V, const Plan& L, double ptol, int prec,
                               uint32_t idx, const Tables& T, uint32_t group,
                               unsigned long long* __restrict__ fb_list,
-                              uint32_t* __restrict__ fb_count, bool filter) {
+                              uint32_t* __restrict__ fb_count, WordTables what) {
   const bool df = prec == KL_DF64;
-  const uint32_t nP = 4u * L.nr;
-  if (idx >= nP) {
-    const uint32_t slot = idx - nP;
-    double2 v;
-    if (L.so == 0) {
-      v = T.Sit[slot];
-    } else {
-      const int u = (int)(slot / L.ns);
-      const uint32_t j = slot % L.ns;
-      const uint32_t j_so = j / L.p3_si, rem = j % L.p3_si;
-      const PartM& S = T.Sot[(uint32_t)u * L.p3_so1 + j_so];
-      const int z = allowed_letter((int)(rem / L.p3_si1), (S.edge + 2) & 3);
-      const double2 t = T.Sit[(uint32_t)z * L.p3_si1 + rem % L.p3_si1];
-      const dc r = mobius(S.m, {t.x, t.y});
-      v = make_double2(r.re, r.im);
-    }
-    T.suf64[slot] = v;
-    // pair-interleaved FP32 table: per first letter u, entry k holds
-    // (re v_2k, re v_2k+1, im v_2k, im v_2k+1); an odd count is padded with NaN
-    const uint32_t u = slot / L.ns, j = slot % L.ns;
-    float* e = (float*)T.suf32p + 4ull * ((uint64_t)u * L.npairs + j / 2u);
-    e[j & 1u] = (float)v.x;
-    e[2 + (j & 1u)] = (float)v.y;
-    if (j + 1u == L.ns && (L.ns & 1u)) {
-      e[1] = __int_as_float(0x7FC00000);
-      e[3] = __int_as_float(0x7FC00000);
-    }
-    if (df) {
-      // pair-interleaved double-float table, padded with NaN like the FP32 one
-      float* q = (float*)T.sufdf + 8ull * ((uint64_t)u * L.npairs + j / 2u);
-      float rh, rl, ih, il;
-      split_df(v.x, rh, rl);
-      split_df(v.y, ih, il);
-      q[j & 1u] = rh;
-      q[2 + (j & 1u)] = rl;
-      q[4 + (j & 1u)] = ih;
-      q[6 + (j & 1u)] = il;
-      if (j + 1u == L.ns && (L.ns & 1u))
-        for (int c = 1; c < 8; c += 2) q[c] = __int_as_float(0x7FC00000);
-    }
+  if (idx >= 4u * L.nr) {
+    suffix_entry(L, prec, idx - 4u * L.nr, T);
     return;
   }
   const int x = (int)(idx / L.nr);
@@ -682,22 +705,21 @@ __device__ void combine_entry(const View& V, const Plan& L, double ptol, int pre
   const uint32_t slot = (uint32_t)x * L.np + r;
   PrefixRec R;
   prefix_rec(V, L, ptol, prec, T, x, r, R);
-  if (R.fl & kFallback) {
+  if (what == kPlainTables && (R.fl & kFallback)) {
     const uint32_t k = atomicAdd(fb_count, 1u);
     fb_list[k] = ((unsigned long long)group << 32) | slot;
   }
   T.pre64[slot] = R.c64;
   if (df && !(R.fl & kDirect)) T.predf[slot] = R.cd;
-  // prefixes on the FP32 map need its record, the others their filter
-  // constants in its place (kl_filter.cuh)
-  if (R.fl & kOnFp32) {
-    T.pre32[slot] = R.c32;
-  } else if (filter) {
+  if (what == kFilterTables) {
     PreF cf;
     if (!(R.fl & kDirect) && filter_consts(V, R.c64, cf))
       *filter_slot(T, slot) = cf;
     else
       R.fl |= kNoFilter;
+  } else {
+    if (what == kCullTables && !(R.fl & (kOnFp32 | kDirect | kWide))) R.fl |= kNear32;
+    if (R.fl & (kOnFp32 | kNear32)) T.pre32[slot] = pre32_of(R.c64);
   }
   T.flags[slot] = R.fl;
 }

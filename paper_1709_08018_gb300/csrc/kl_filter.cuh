@@ -75,6 +75,16 @@ __device__ __forceinline__ int exact_pixel(const Tables& T, const View& V, uint3
     const uint32_t col = ua - 0x4B400000u, row = va - 0x4B400000u;
     return (col < V.W && row < V.H) ? (int)(row * V.W + col) : -1;
   }
+  if (PREC == KL_MIXED && (fl & kOnFp32)) {
+    const Pre32 k = pre32_of(T.pre64[slot]);
+    const float4 s = __ldg(T.suf32p + (size_t)u * npairs + j / 2u);
+    const bool odd = j & 1u;
+    float uf, vf;
+    uv_pole32(k, odd ? s.y : s.x, odd ? s.w : s.z, uf, vf);
+    const int col = __float_as_int(__fadd_rd(uf, 12582912.0f)) - k.kx;
+    const int row = __float_as_int(__fadd_rd(vf, 12582912.0f)) - k.ky;
+    return ((uint32_t)col < V.W && (uint32_t)row < V.H) ? row * (int)V.W + col : -1;
+  }
   const double2 s = __ldg(T.suf64 + (size_t)u * ns + j);
   double uu, vv;
   if (fl & kDirect)

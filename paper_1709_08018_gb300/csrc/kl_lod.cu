@@ -620,7 +620,7 @@ __global__ void lod_combine_kernel(View V, Plan L, double ptol, int mixed, Table
   const uint32_t total = combine_count(L);
   for (uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total;
        idx += gridDim.x * blockDim.x)
-    combine_entry(V, L, ptol, mixed, idx, T, 0u, T.fb, T.fbcount, false);
+    combine_entry(V, L, ptol, mixed, idx, T, 0u, T.fb, T.fbcount, kPlainTables);
 }
 
 // The pruned render needs the prefix constants of the deferred level-hi
@@ -633,7 +633,7 @@ __global__ void lod_combine_listed_kernel(View V, Plan L, double ptol, int mixed
   for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += gridDim.x * blockDim.x) {
     const uint32_t idx = e < n ? slots[e] : 4u * L.np + (e - n);
-    combine_entry(V, L, ptol, mixed, idx, T, 0u, T.fb, T.fbcount, false);
+    combine_entry(V, L, ptol, mixed, idx, T, 0u, T.fb, T.fbcount, kCullTables);
   }
 }
 

@@ -5,6 +5,7 @@
 #include <mutex>
 
 #include "kl_common.cuh"
+#include "kl_tiling.cuh"
 
 namespace {
 
@@ -47,13 +48,13 @@ __global__ void parts_kernel(Group G, Plan L, int renorm, Tables T, Clear C,
 // Entries [first, combine_count): first = 4 nr (the prefixes skipped) when
 // the prefix tables are already in place.
 __global__ void combine_kernel(View V, Plan L, double ptol, int prec, Tables T, uint32_t first,
-                               int filter) {
+                               WordTables what) {
   pdl_trigger();
   pdl_wait();
   const uint32_t total = combine_count(L);
   for (uint32_t idx = first + blockIdx.x * blockDim.x + threadIdx.x; idx < total;
        idx += gridDim.x * blockDim.x)
-    combine_entry(V, L, ptol, prec, idx, T, 0u, T.fb, T.fbcount, filter != 0);
+    combine_entry(V, L, ptol, prec, idx, T, 0u, T.fb, T.fbcount, what);
 }
 
 // ---------------------------------------------------------------------------
@@ -193,49 +194,6 @@ __global__ void render_single_letter_kernel(Group G, View V, uint32_t* img,
   }
 }
 
-// Tiling mode, the short lengths 1..k0: one thread per node, its word
-// decoded from the node's index within its length and evaluated point by
-// point from the inside out (the seed of w_k, then the maps of w_k, ..., w_1),
-// in FP64 with a refined reciprocal instead of division.  These lengths hold
-// few words (2 (3^k0 - 1)), so one launch for all of them replaces a render
-// per length, whose launches would cost more than its words.
-constexpr uint32_t kShortTiling = 9;
-
-__global__ void tiling_short_kernel(Group G, View V, uint32_t k0, int fp64_count,
-                                    uint32_t* __restrict__ img, unsigned long long* counters) {
-  uint64_t total = 0, nk = 4;
-  for (uint32_t k = 1; k <= k0; ++k, nk *= 3) total += nk;
-  uint32_t in_window = 0, words = 0, atomics = 0;
-  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < total;
-       i += (uint64_t)gridDim.x * blockDim.x) {
-    uint64_t r = i, n = 4;
-    uint32_t k = 1;
-    while (r >= n) {
-      r -= n;
-      n *= 3;
-      ++k;
-    }
-    int w[kShortTiling];
-    decode_word(r, (int)k, w);
-    dc z = {G.seed[2 * w[k - 1]], G.seed[2 * w[k - 1] + 1]};
-    for (int j = (int)k - 1; j >= 0; --j) {
-      const double* M = G.g + 8 * w[j];
-      const dc num = {M[0] * z.re - M[1] * z.im + M[2], M[0] * z.im + M[1] * z.re + M[3]};
-      const dc den = {M[4] * z.re - M[5] * z.im + M[6], M[4] * z.im + M[5] * z.re + M[7]};
-      const double rc = rcp64(den.re * den.re + den.im * den.im);
-      z = {(num.re * den.re + num.im * den.im) * rc, (num.im * den.re - num.re * den.im) * rc};
-    }
-    const int pix = pixel64((z.re - V.x0) * V.sx, (V.y1 - z.im) * V.sy, V);
-    ++words;
-    if (pix >= 0) {
-      atomicAdd(img + pix, 1u);
-      ++in_window;
-      ++atomics;
-    }
-  }
-  publish_counts(in_window, words, fp64_count ? words : 0u, atomics, counters);
-}
-
 __global__ void eval_kernel(const uint64_t* __restrict__ idx, uint64_t n, uint64_t N, Group G,
                             Plan L, View V, int prec, Tables T, double* __restrict__ out) {
   const bool mixed = prec == KL_MIXED, df = prec == KL_DF64;
@@ -312,41 +270,33 @@ int prof_mark(cudaEvent_t e, cudaStream_t s) {
   return cudaEventRecord(e, s) == cudaSuccess ? KL_OK : KL_ECUDA;
 }
 
+// 32-thread blocks that clear C's image with 16-byte stores.
+uint32_t clear_blocks(const Clear& C, int sms) {
+  if (!C.words) return 0u;
+  const size_t need = (C.words / 4 + 31) / 32;
+  return (uint32_t)(need < (size_t)sms * 8 ? (need > 0 ? need : 1) : (size_t)sms * 8);
+}
+
 // Tables of a render: parts (with the image clearing of C riding along),
 // then combine, launched as a programmatic dependent of parts.
 // The tables of plan L; with prefix_ready the prefix tables (and the list of
 // fallback prefixes) are taken as they are and only the suffix side is built.
 int build_tables(const kl_params* p, const Plan& L, const View& V, const Group& G,
                  const Tables& T, cudaStream_t st, const Clear& C = Clear{},
-                 bool prefix_ready = false, bool filter = false) {
+                 bool prefix_ready = false, WordTables what = kPlainTables) {
   const int prec = (int)p->precision;
   const uint32_t first_part = prefix_ready ? 4u * L.p3_q1 + (L.p > L.q ? 4u * L.p3_pq : 0u) : 0u;
   const uint32_t first_comb = prefix_ready ? 4u * L.nr : 0u;
   const uint32_t nParts = parts_count(L) - first_part;
   const uint32_t part_blocks = nParts > 0 ? (nParts + kPartLanes - 1) / kPartLanes : 1u;
-  uint32_t clear_blocks = 0;
-  if (C.words) {
-    const int sms = sm_count();
-    if (sms <= 0) return KL_ECUDA;
-    const size_t need = (C.words / 4 + 31) / 32;  // 16-byte stores, 32-thread blocks
-    clear_blocks = (uint32_t)(need < (size_t)sms * 8 ? (need > 0 ? need : 1) : (size_t)sms * 8);
-  }
-  parts_kernel<<<part_blocks + clear_blocks, 32, 0, st>>>(G, L, (int)p->renorm_every, T, C,
+  const int sms = sm_count();
+  if (sms <= 0) return KL_ECUDA;
+  parts_kernel<<<part_blocks + clear_blocks(C, sms), 32, 0, st>>>(G, L, (int)p->renorm_every, T, C,
                                                           part_blocks, first_part);
   if (check_launch() != KL_OK) return KL_ECUDA;
   const uint32_t n = combine_count(L) - first_comb;
   return launch_dependent(combine_kernel, dim3(n > 0 ? (n + 127) / 128 : 1u), dim3(128), st, V,
-                          L, p->parabolic_tol, prec, T, first_comb, filter ? 1 : 0);
-}
-
-// Length k of a tiling render of *p: a limit-set render of the words of
-// length k; the caller's prefix length applies to length d only.
-kl_params length_params(const kl_params* p, uint32_t k) {
-  kl_params q = *p;
-  q.depth = k;
-  q.mode = KL_LIMIT_SET;
-  if (k != p->depth) q.prefix_len = 0;
-  return q;
+                          L, p->parabolic_tol, prec, T, first_comb, what);
 }
 
 // Workspace bytes of *p (tiling: the largest over its lengths), or 0.
@@ -516,8 +466,10 @@ int render_length(const kl_params* p, uint32_t* d_image, unsigned long long* cnt
   const Tables T = carve(L, d_workspace);
   Clear C{};
   if (!p->accumulate) C = {d_image, (size_t)p->width * p->height, cnt};
-  const bool filter = p->precision != KL_MIXED && !p->cull;
-  st = build_tables(p, L, V, G, T, s, C, prev && prefix_tables_shared(*prev, L, p), filter);
+  st = build_tables(p, L, V, G, T, s, C, prev && prefix_tables_shared(*prev, L, p),
+                    p->cull                       ? kCullTables
+                    : p->precision == KL_MIXED ? kPlainTables
+                                               : kFilterTables);
   if (st != KL_OK) return st;
   switch (p->block_threads) {
     case 64: return launch_render<64>(p, L, V, T, d_image, cnt, s, profile);
@@ -530,22 +482,74 @@ int render_length(const kl_params* p, uint32_t* d_image, unsigned long long* cnt
 
 namespace {
 
-// A tiling render of *p (already validated): the lengths above kShortTiling
-// as renders of their own, the longest first (it clears the image unless
-// accumulating), each next one added in; then all the short lengths in one
-// launch.  Consecutive lengths with the same prefix length share its prefix
-// tables, built once.
+using TilingKernel = void (*)(Group, View, LengthSet, uint32_t*, unsigned long long*);
+
+template <int BT>
+TilingKernel tiling_kernel(uint32_t precision) {
+  switch (precision) {
+    case KL_FP64: return tiling_words_kernel<BT, KL_FP64>;
+    case KL_DF64: return tiling_words_kernel<BT, KL_DF64>;
+    default: return tiling_words_kernel<BT, KL_MIXED>;
+  }
+}
+
+// Lengths k, k - 1, ... of *p that share prefix tables, and the lengths up to
+// k0, in three launches.  *next: the first length not rendered (k: none was;
+// the lengths do not go together).
+int render_lengths(const kl_params* p, uint32_t k, uint32_t k0, uint32_t* d_image,
+                   unsigned long long* cnt, void* d_workspace, cudaStream_t s, uint32_t* next) {
+  const uint32_t bt = p->block_threads ? p->block_threads : (uint32_t)kDefaultThreads;
+  const TilingKernel kern = bt == 64    ? tiling_kernel<64>(p->precision)
+                            : bt == 256 ? tiling_kernel<256>(p->precision)
+                                        : tiling_kernel<128>(p->precision);
+  *next = k;
+  int sms = 0, occ = 0;
+  if (device_slots((const void*)kern, (int)bt, &sms, &occ) != KL_OK) return KL_ECUDA;
+  LengthSet S;
+  const int st = make_lengths(p, k, k0, d_workspace, sms * occ * (int)(bt / 32), &S);
+  if (st != KL_OK) return st;
+  if (S.n < 2 || k - S.n > k0) return KL_OK;  // only a set that reaches the short lengths
+  const View V = make_view(p);
+  const Group G = make_group(p);
+  Clear C{};
+  if (!p->accumulate && k == p->depth) C = {d_image, (size_t)p->width * p->height, cnt};
+  const uint32_t part_blocks = (S.parts[S.n] + kPartLanes - 1) / kPartLanes;
+  tiling_parts_kernel<<<part_blocks + clear_blocks(C, sms), 32, 0, s>>>(
+      G, S, (int)p->renorm_every, C, part_blocks, kPartLanes);
+  if (check_launch() != KL_OK) return KL_ECUDA;
+  if (launch_dependent(tiling_combine_kernel, dim3((S.comb[S.n] + 127) / 128), dim3(128), s, V, S,
+                       p->parabolic_tol, (int)p->precision) != KL_OK)
+    return KL_ECUDA;
+  const bool profile = k == p->depth;
+  if (profile && prof_mark(g_prof_start, s) != KL_OK) return KL_ECUDA;
+  if (launch_dependent(kern, dim3((unsigned)(sms * occ)), dim3(bt), s, G, V, S, d_image, cnt) !=
+      KL_OK)
+    return KL_ECUDA;
+  *next = k0;
+  return profile ? prof_mark(g_prof_stop, s) : KL_OK;
+}
+
+// A tiling render of *p (already validated): the lengths above kShortTiling,
+// the longest first (it clears the image unless accumulating), each next one
+// added in, then the short ones.  The lengths that share their prefix tables
+// and reach the short ones go together (lengths 10 .. 17 of the default plans);
+// longer ones, culled ones and a caller's prefix length are renders of their
+// own, consecutive ones with the same prefix length sharing its tables.
 int render_tiling(const kl_params* p, uint32_t* d_image, unsigned long long* cnt,
                   void* d_workspace, cudaStream_t s) {
   const uint32_t k0 = p->depth < kShortTiling ? p->depth : kShortTiling;
   Plan prev;
   bool have_prev = false;
   for (uint32_t k = p->depth; k > k0; --k) {
+    uint32_t next = k;
+    int st = render_lengths(p, k, k0, d_image, cnt, d_workspace, s, &next);
+    if (st != KL_OK) return st;
+    if (next == k0) return KL_OK;
     kl_params q = length_params(p, k);
     q.accumulate = k == p->depth ? p->accumulate : 1u;
     Plan used;
-    const int st = render_length(&q, d_image, cnt, d_workspace, s, k == p->depth,
-                                 have_prev ? &prev : nullptr, &used);
+    st = render_length(&q, d_image, cnt, d_workspace, s, k == p->depth,
+                       have_prev ? &prev : nullptr, &used);
     if (st != KL_OK) return st;
     prev = used;
     have_prev = used.d > 1;
@@ -557,10 +561,8 @@ int render_tiling(const kl_params* p, uint32_t* d_image, unsigned long long* cnt
     if (cnt && cudaMemsetAsync(cnt, 0, KL_N_COUNTERS * sizeof(uint64_t), s) != cudaSuccess)
       return KL_ECUDA;
   }
-  const int sms = sm_count();
-  if (sms <= 0) return KL_ECUDA;
-  tiling_short_kernel<<<sms * 4, 256, 0, s>>>(make_group(p), make_view(p), k0,
-                                              p->precision != KL_FP64, d_image, cnt);
+  tiling_short_kernel<<<(short_roots(k0) + 31) / 32, 32, 0, s>>>(
+      make_group(p), make_view(p), k0, p->precision != KL_FP64, d_image, cnt);
   return check_launch();
 }
 
