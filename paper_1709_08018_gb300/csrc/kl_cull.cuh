@@ -53,6 +53,12 @@ constexpr int kUncertified = -2;
 // pixel, is far above the per-word map's rounding error; the interval ends are
 // rounded outwards before flooring, so a certified block never straddles a
 // pixel edge.
+//
+// EXACT64: the block of a prefix whose words run in FP64 (k: its constants
+// rounded to FP32, D already widened by near_slack).  The rounding of the other
+// constants and of this test's own steps is below 16 eps of |M| / |w|, both
+// axes alike, eps = 2^-24; the code takes 32.
+template <bool EXACT64 = false>
 __device__ __forceinline__ int block_pixel32(const Pre32& k, float nrm, float4 D, const View& V) {
   const float c0r = D.x + k.gr, c0i = D.y + k.gi;
   const float n2 = fmaf(c0r, c0r, c0i * c0i), rho2 = D.z * D.z;
@@ -61,7 +67,11 @@ __device__ __forceinline__ int block_pixel32(const Pre32& k, float nrm, float4 D
   const float X = fmaf(fmaf(k.c1, c0r, k.c2 * c0i), rq, k.axf);
   const float Y = fmaf(fmaf(k.c3, c0r, k.c4 * c0i), rq, k.ayf);
   const float R = nrm * D.z * rq;
-  const float m = R + fmaf(fabsf(X) + fabsf(Y) + R, 0x1p-20f, 0x1p-11f);
+  float m = R + fmaf(fabsf(X) + fabsf(Y) + R, 0x1p-20f, 0x1p-11f);
+  if (EXACT64) {
+    if (!(n2 > 1e-30f && n2 < 1e30f)) return kUncertified;
+    m = fmaf(nrm * sqrtf(n2) * rq, 0x1p-19f, m);
+  }
   if (m < 0.5f && fabsf(X) < 0x1p21f && fabsf(Y) < 0x1p21f) {
     const float magic = 12582912.0f;  // 1.5 * 2^23: t bits - 0x4B400000 = floor
     const int xl = __float_as_int(__fadd_rd(__fsub_rd(X, m), magic));
@@ -80,6 +90,13 @@ __device__ __forceinline__ int block_pixel32(const Pre32& k, float nrm, float4 D
       Ya - m > (float)V.H + 1.0f)
     return -1;
   return kUncertified;
+}
+
+// What an FP32 test of an FP64 block adds to the disk's radius: the distance
+// from v + gamma to the sum of the two rounded to FP32 is below 2^-24 of |v| +
+// |gamma| per part; four times that.
+__device__ __forceinline__ float near_slack(const Pre32& k, const float4& D) {
+  return 0x1p-22f * (fabsf(k.gr) + fabsf(k.gi) + fabsf(D.x) + fabsf(D.y) + D.z);
 }
 
 // The same in FP64 (pole-form prefixes; absolute pixel coordinates).  Margin
@@ -140,6 +157,49 @@ __device__ __forceinline__ void mixed_block_words(uint32_t slot, int u, uint32_t
     ++words;
   }
   if (j1 > j0) mixed_slot_words(slot, u, j0 / 2u, j1 / 2u, L, V, T, t, words, img);
+}
+
+// FP64 words of a pole-form prefix on suffix points [j0, j1): each in FP32 first
+// (k: the prefix's constants rounded to FP32), in FP64 where the bound does not
+// settle the pixel, so every word lands where FP64 puts it.  Error, R = |M| / |w|
+// an upper bound on both parts of the offset from alpha, q = (|v| + |gamma|) /
+// |w|: the rounded sum w is off by eps (1 + q) |w|, which moves the offset by at
+// most twice that of R; rounding M, the products, |w|^2, its reciprocal root and
+// the last products, 18 eps R; the sum with alpha, eps of its parts.  Below eps R
+// (22 + 2 q) in all; the code takes eps R (64 + 8 q), and settles nothing where
+// 8 eps q >= 1/4.
+__device__ __forceinline__ void near_words64(const Pre32& k, const Pre64* __restrict__ c64,
+                                             float nrm, const float4* s32, const double2* s64,
+                                             uint32_t j0, uint32_t j1, const View& V, Tally& t,
+                                             uint32_t* __restrict__ img) {
+  const float c0 = 4.0f * kEps24 * (2.0f + fabsf(k.axf) + fabsf(k.ayf));
+  const float ag = fabsf(k.gr) + fabsf(k.gi), magic = 12582912.0f;
+  for (uint32_t j = j0; j < j1; ++j) {
+    const float4 s = __ldg(s32 + j / 2u);
+    const float vr = j & 1u ? s.y : s.x, vi = j & 1u ? s.w : s.z;
+    const float wr = vr + k.gr, wi = vi + k.gi;
+    const float m = fmaf(wr, wr, wi * wi), rw = rsqrtf(m), r = rw * rw;
+    const float X = fmaf(k.c1, wr, k.c2 * wi) * r, Y = fmaf(k.c3, wr, k.c4 * wi) * r;
+    const float q = 8.0f * kEps24 * (ag + fabsf(vr) + fabsf(vi)) * rw;
+    const float E = fmaf(nrm * rw, q + 64.0f * kEps24, c0);
+    const float u = X + k.axf, v = Y + k.ayf;
+    const int ul = __float_as_int(__fadd_rd(u - E, magic));
+    const int uh = __float_as_int(__fadd_rd(u + E, magic));
+    const int vl = __float_as_int(__fadd_rd(v - E, magic));
+    const int vh = __float_as_int(__fadd_rd(v + E, magic));
+    int pix;
+    if (m > 1e-30f && m < 1e30f && q < 0.25f && E < 0.25f && fabsf(u) < 0x1p20f && fabsf(v) < 0x1p20f && ul == uh &&
+        vl == vh) {
+      const int col = ul - k.kx, row = vl - k.ky;
+      pix = ((uint32_t)col < V.W && (uint32_t)row < V.H) ? row * (int)V.W + col : -1;
+    } else {
+      const double2 z = __ldg(s64 + j);
+      double uu, vv;
+      uv_pole64(*c64, z.x, z.y, uu, vv);
+      pix = pixel64(uu, vv, V);
+    }
+    t.add(pix, img);
+  }
 }
 
 // Disk of culling block `disk` of plan L (all lanes of a warp take part),
@@ -323,6 +383,12 @@ struct CullWarp {
     const uint32_t j0 = b * C->sz[l];
     if (MIXED && !f64) {
       mixed_block_words(slot, (int)u, j0, C->sz[l], L, V, T, t, words, img);
+    } else if (T.flags[slot] & kNear32) {
+      near_words64(T.pre32[slot], T.pre64 + slot, T.nrm32[slot],
+                   T.suf32p + (size_t)u * L.npairs, T.suf64 + (size_t)u * L.ns, j0,
+                   j0 + C->sz[l], V, t, img);
+      words += C->sz[l];
+      if (MIXED) fp64_words += C->sz[l];
     } else {
       words64(T.pre64[slot], T.flags[slot] & kDirect, T.suf64 + (size_t)u * L.ns, j0,
               j0 + C->sz[l], V, t, img);
@@ -345,7 +411,18 @@ struct CullWarp {
                                       uint32_t l, bool f64, uint32_t b) {
     const uint32_t di = C->disk[l] + u * C->nb[l] + b;
     if (MIXED && !f64) return block_pixel32(T.pre32[slot], T.nrm32[slot], T.disk32[di], V);
-    if (T.flags[slot] & kDirect) return kUncertified;
+    const uint32_t fl = T.flags[slot];
+    if (fl & kDirect) return kUncertified;
+    if (fl & kNear32) {
+      // in FP32 unless rounding v and gamma would more than double the disk
+      const Pre32 k = T.pre32[slot];
+      float4 D = T.disk32[di];
+      const float slack = near_slack(k, D);
+      if (slack < D.z) {
+        D.z += slack;
+        return block_pixel32<true>(k, T.nrm32[slot], D, V);
+      }
+    }
     return block_pixel64(T.pre64[slot], T.nrm64[slot], T.disk64[di], V);
   }
   // the outcome of one test per lane (act: this lane tested an entry)
@@ -418,6 +495,21 @@ struct CullWarp {
   }
 };
 
+// Order of a culled render's prefix blocks.  A prefix whose outer letters are
+// one long run (a^8 x, B^8 x, b^8 x, A^8 x) covers a large piece of the image:
+// none of its blocks is certified before the smallest, and an item of such
+// prefixes takes a warp a third of the whole render's time.  Their slots are the
+// first, the last and the middle ones of a letter (base-3 digits all 0, 2 or 1),
+// so those blocks of all letters are drawn first; in slot order the last block
+// of the last letter ran on alone at the end.
+__device__ __forceinline__ uint32_t cull_block_order(uint32_t i, uint32_t n) {
+  if (i == 0 || n < 4) return i;
+  const uint32_t mid = (n - 1) / 2;
+  if (i == 1) return n - 1;
+  if (i == 2) return mid;
+  return i - 2 + (i - 2 >= mid ? 1u : 0u);
+}
+
 // The lanes of one culling item: prefix slot of this lane and whether it is
 // live, and (mixed) whether it takes the FP64 path.  Items are 32 prefixes x
 // a chunk of top-level blocks of one suffix letter.
@@ -425,9 +517,11 @@ template <bool MIXED>
 __device__ __forceinline__ void cull_item(CullWarp<MIXED>& w, uint32_t item, const Work& Wk,
                                           const Plan& L, const View& V, const Tables& T,
                                           uint32_t* __restrict__ img, uint32_t top_blocks) {
-  int x, u;
-  uint32_t pb, c;
-  item_of(item, Wk, x, u, pb, c);
+  // prefix blocks slowest, suffix blocks fastest
+  const uint32_t c = item % Wk.n_chunks, t = item / Wk.n_chunks;
+  const uint32_t q = t % 12u, pb = cull_block_order(t / 12u, Wk.n_pb);
+  const int x = (int)(q / 3u);
+  const int u = allowed_letter((int)(q % 3u), (x + 2) & 3);
   const uint32_t k = pb * 32 + w.lane;
   const uint32_t slot = (uint32_t)x * L.np + L.r0 + k;
   const bool live = k < L.nr;
