@@ -299,9 +299,11 @@ __device__ __forceinline__ int guarded_pixel_df(D1 u, D1 v, const View& V, float
   return (int)cv * (int)V.W + (int)cu;
 }
 
-__global__ void vstar_kernel(Group G, int D, int lo, int hi, double2* vstar) {
-  const int x = threadIdx.x & 3, e = (threadIdx.x >> 2) % kReps;
-  const int k = lo + (threadIdx.x >> 2) / kReps;
+// Entry i of vstar: representative e of letter x at level k.
+__device__ __noinline__ void vstar_entry(const Group& G, int D, int lo, int hi, uint32_t i,
+                                         double2* vstar) {
+  const int x = (int)(i & 3u), e = (int)(i >> 2) % kReps;
+  const int k = lo + (int)(i >> 2) / kReps;
   if (k > hi) return;
   const int m = D - k;
   int w[KL_MAX_DEPTH];
@@ -315,16 +317,45 @@ __global__ void vstar_kernel(Group G, int D, int lo, int hi, double2* vstar) {
   vstar[(e * 4 + x) * (hi + 1) + k] = make_double2(z.re, z.im);
 }
 
-__global__ void init_active_kernel(Group G, int k, uint32_t nk, Active* out, uint32_t* count) {
-  const uint32_t n = 4u * nk;
-  for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
-    Active a;
-    m1_store(m1_of(node_matrix(G, k, s, nk)), a);
-    a.slot = s;
-    a.pad[0] = a.pad[1] = a.pad[2] = 0;
-    out[s] = a;
+// The pruned render's first launch: vstar, the parts tables of its exact render
+// and the active nodes of level lo, `lanes` entries to a block (each is a chain
+// of dependent FP64 operations; a few thousand are better spread over the SMs,
+// 16 to a block, than packed into warps), the counters, and the image cleared by
+// the blocks after them.  As four memsets and three kernels one after the other these took 90 us
+// (depth 22, 8192^2), now the 45 us of clearing the image; the whole render 742 ->
+// 692 us.  (The kernels after it as programmatic dependents: 841 us.  Early blocks
+// hold the shared memory that the level before them still needs.)
+__global__ void __launch_bounds__(32) lod_begin_kernel(
+    const __grid_constant__ Group G, const __grid_constant__ Plan L, int renorm, Tables T, int D,
+    int lo, int hi, uint32_t nk, double2* vstar, Active* act, uint32_t* counts,
+    unsigned long long* stats, Clear C, uint32_t entry_blocks, uint32_t lanes) {
+  if (blockIdx.x >= entry_blocks) {
+    clear_words(C.img, C.words, (size_t)(blockIdx.x - entry_blocks) * blockDim.x + threadIdx.x,
+                (size_t)(gridDim.x - entry_blocks) * blockDim.x);
+    return;
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) *count = n;
+  if (blockIdx.x == 0) {
+    const uint32_t t = threadIdx.x;
+    counts[t] = t == (uint32_t)lo ? 4u * nk : 0u;
+    counts[32 + t] = 0u;
+    if (t < 4) stats[t] = 0ull;
+    if (t < KL_N_COUNTERS) C.counters[t] = 0ull;
+    if (t < 2) T.fbcount[t] = 0u;
+  }
+  if (threadIdx.x >= lanes) return;
+  uint32_t i = blockIdx.x * lanes + threadIdx.x;
+  const uint32_t nv = 4u * kReps * (uint32_t)(hi - lo + 1), np = parts_count(L);
+  if (i < nv) {
+    vstar_entry(G, D, lo, hi, i, vstar);
+  } else if ((i -= nv) < np) {
+    part_entry(G, L, renorm, i, T);
+  } else if ((i -= np) < 4u * nk) {
+    Active a;
+    m1_store(m1_of(node_matrix(G, lo, i, nk)), a);
+    a.slot = i;
+    a.pad[0] = a.pad[1] = a.pad[2] = 0;
+    act[i] = a;
+  }
 }
 
 // One level: each CTA takes tiles of 128 active nodes (thread t: node t of
@@ -598,10 +629,6 @@ RenderLayout render_layout(const LodPlan& P, const Plan& L) {
   return Y;
 }
 
-int build_tables_forced(const kl_params* p, const Plan& L, const View& V, const Group& G,
-                        const Tables& T, cudaStream_t st, const uint32_t* slots,
-                        const uint32_t* n_slots);
-
 unsigned grid_for(uint64_t n, int threads, int cap_per_sm) {
   const int sms = sm_count();
   const uint64_t b = (n + threads - 1) / threads;
@@ -637,20 +664,13 @@ __global__ void lod_combine_listed_kernel(View V, Plan L, double ptol, int mixed
   }
 }
 
-// Tables of *p for the split (prefix hi, suffix D - hi): every prefix slot,
-// or, with `slots`, only the listed ones.
+// Tables of *p for the split (prefix hi, suffix D - hi).
 int build_tables_forced(const kl_params* p, const Plan& L, const View& V, const Group& G,
-                        const Tables& T, cudaStream_t st, const uint32_t* slots,
-                        const uint32_t* n_slots) {
+                        const Tables& T, cudaStream_t st) {
   if (cudaMemsetAsync(T.fbcount, 0, 2 * sizeof(uint32_t), st) != cudaSuccess) return KL_ECUDA;
   const uint32_t nParts = parts_count(L);
   lod_parts_kernel<<<(nParts + 31) / 32, 32, 0, st>>>(G, L, (int)p->renorm_every, T);
   if (check_launch() != KL_OK) return KL_ECUDA;
-  if (slots) {
-    lod_combine_listed_kernel<<<grid_for(combine_count(L), 128, 8), 128, 0, st>>>(
-        V, L, p->parabolic_tol, p->precision == KL_MIXED, T, slots, n_slots);
-    return check_launch();
-  }
   const uint32_t n = combine_count(L);
   lod_combine_kernel<<<(n + 127) / 128, 128, 0, st>>>(V, L, p->parabolic_tol,
                                                        p->precision == KL_MIXED, T);
@@ -705,7 +725,7 @@ extern "C" int kl_lod_labels(const kl_params* p, uint32_t lo, uint32_t hi, float
     return KL_ECUDA;
   box_init_kernel<<<grid_for(nh, 256, 8), 256, 0, s>>>(B, nh);
   if (check_launch() != KL_OK) return KL_ECUDA;
-  st = build_tables_forced(&q, L, V, G, T, s, nullptr, nullptr);
+  st = build_tables_forced(&q, L, V, G, T, s);
   if (st != KL_OK) return st;
   int sms = 0, occ = 0;
   const bool mixed = p->precision == KL_MIXED;
@@ -777,8 +797,6 @@ int render_lod_impl(const kl_params* p, uint32_t lo, uint32_t hi, const float* d
   char* ws = (char*)d_workspace;
   const View V = make_view(p);
   const Group G = make_group(p);
-  kl_params q = *p;
-  q.prefix_len = hi;
   const Tables T = carve(L, ws + Y.tables);
   double2* vstar = (double2*)(ws + Y.vstar);
   Active* act[2] = {(Active*)(ws + Y.act0), (Active*)(ws + Y.act1)};
@@ -786,16 +804,20 @@ int render_lod_impl(const kl_params* p, uint32_t lo, uint32_t hi, const float* d
   uint32_t* counts = (uint32_t*)(ws + Y.counts);  // [k]: active count of level k, [32]: deferred
   unsigned long long* cnt = (unsigned long long*)d_counters;
   unsigned long long* stats = (unsigned long long*)d_stats;
-  if (cudaMemsetAsync(d_image, 0, (size_t)p->width * p->height * sizeof(uint32_t), s) !=
-          cudaSuccess ||
-      cudaMemsetAsync(cnt, 0, KL_N_COUNTERS * sizeof(uint64_t), s) != cudaSuccess ||
-      cudaMemsetAsync(stats, 0, 4 * sizeof(uint64_t), s) != cudaSuccess ||
-      cudaMemsetAsync(counts, 0, 64 * sizeof(uint32_t), s) != cudaSuccess)
+  int sms = 0, occ = 0;
+  if (device_slots((const void*)lod_cull_kernel<128, true>, 128, &sms, &occ) != KL_OK)
     return KL_ECUDA;
-  vstar_kernel<<<1, 4 * kReps * (kMaxPrefix + 1), 0, s>>>(G, P.D, P.lo, P.hi, vstar);
-  if (check_launch() != KL_OK) return KL_ECUDA;
-  init_active_kernel<<<grid_for(4ull * P.p3[lo], 128, 8), 128, 0, s>>>(G, (int)lo, P.p3[lo],
-                                                                        act[0], counts + lo);
+  const size_t words = (size_t)p->width * p->height, need = (words / 4 + 31) / 32;
+  const Clear C = {d_image, words, cnt};
+  const uint32_t clear = (uint32_t)(need < (size_t)sms * 8 ? (need > 0 ? need : 1)
+                                                           : (size_t)sms * 8);
+  const uint32_t entries =
+      4u * kReps * (uint32_t)(P.hi - P.lo + 1) + parts_count(L) + 4u * P.p3[lo];
+  const uint32_t lanes = entries < 65536u ? 16u : 32u;
+  const uint32_t entry_blocks = (entries + lanes - 1) / lanes;
+  lod_begin_kernel<<<entry_blocks + clear, 32, 0, s>>>(
+      G, L, (int)p->renorm_every, T, P.D, P.lo, P.hi, P.p3[lo], vstar, act[0], counts, stats, C,
+      entry_blocks, lanes);
   if (check_launch() != KL_OK) return KL_ECUDA;
   if (d_mlp && cudaFuncSetAttribute(expand_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)kFwdSmem) != cudaSuccess)
@@ -809,11 +831,10 @@ int render_lod_impl(const kl_params* p, uint32_t lo, uint32_t hi, const float* d
         counts + k + 1, deferred, counts + 32, d_image, cnt, stats);
     if (check_launch() != KL_OK) return KL_ECUDA;
   }
-  st = build_tables_forced(&q, L, V, G, T, s, deferred, counts + 32);
-  if (st != KL_OK) return st;
-  int sms = 0, occ = 0;
-  if (device_slots((const void*)lod_cull_kernel<128, true>, 128, &sms, &occ) != KL_OK)
-    return KL_ECUDA;
+  // the prefix constants of the deferred nodes and every suffix point
+  lod_combine_listed_kernel<<<grid_for(combine_count(L), 128, 8), 128, 0, s>>>(
+      V, L, p->parabolic_tol, p->precision == KL_MIXED, T, deferred, counts + 32);
+  if (check_launch() != KL_OK) return KL_ECUDA;
   // block disks (four warps per block), then the deferred prefixes' norms
   const uint32_t small = cull_small_disks(L);
   const uint32_t disk_warps = (small + 31) / 32 + (L.ndisks - small);
