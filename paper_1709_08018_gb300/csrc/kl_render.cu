@@ -110,16 +110,16 @@ __global__ void __launch_bounds__(BT, 1024 / BT) render_words_kernel(
     unsigned long long* counters) {
   __shared__ WarpQueue s_queue[BT / 32];
   __shared__ ExactCtx C;
+  __shared__ unsigned long long s_counts[KL_N_COUNTERS];
   if (threadIdx.x == 0) C = {T, V, L.ns, L.npairs, img};
-  __syncthreads();
+  block_counts_begin(s_counts);
   pdl_wait();
   WordWarp<PREC> w(&C, &s_queue[threadIdx.x >> 5]);
-  for (;;) {
-    const uint32_t item = next_item_warp(T.fbcount + 1);
-    if (item >= Wk.n_items) break;
+  for (uint32_t item = first_item_warp(); item < Wk.n_items;
+       item = later_item_warp(T.fbcount + 1, Wk.n_items))
     word_item(w, item, Wk, L, V, T, img);
-  }
-  w.finish(counters);
+  w.finish(s_counts);
+  block_counts_end(s_counts, counters);
 }
 
 // ---------------------------------------------------------------------------
@@ -348,6 +348,13 @@ WordsKernel words_kernel(uint32_t precision) {
   }
 }
 
+// Persistent blocks for the items of Wk: the resident ones, or fewer where not
+// every warp of them would get an item.
+dim3 words_grid(const Work& Wk, int slots, int bt) {
+  const uint32_t need = (Wk.n_items + bt / 32 - 1) / (bt / 32);
+  return dim3(need < 1 ? 1 : need < (uint32_t)slots ? need : (uint32_t)slots);
+}
+
 template <int BT>
 int launch_render(const kl_params* p, const Plan& L, const View& V, const Tables& T,
                   uint32_t* img, unsigned long long* cnt, cudaStream_t s, bool profile) {
@@ -365,10 +372,11 @@ int launch_render(const kl_params* p, const Plan& L, const View& V, const Tables
     const Work Wk = make_work(L, 32, L.cnb[L.clev - 1], sms * occ * (BT / 32),
                               p->chunk_pairs ? p->chunk_pairs : 1u);
     if (prof_mark(ev0, s) != KL_OK) return KL_ECUDA;
-    const int st = mixed ? launch_dependent(cull_kernel<BT, true>, dim3(sms * occ), dim3(BT), s,
-                                            T, L, V, Wk, img, cnt)
-                         : launch_dependent(cull_kernel<BT, false>, dim3(sms * occ), dim3(BT),
-                                            s, T, L, V, Wk, img, cnt);
+    const dim3 grid = words_grid(Wk, sms * occ, BT);
+    const int st = mixed ? launch_dependent(cull_kernel<BT, true>, grid, dim3(BT), s, T, L, V, Wk,
+                                            img, cnt)
+                         : launch_dependent(cull_kernel<BT, false>, grid, dim3(BT), s, T, L, V,
+                                            Wk, img, cnt);
     if (st != KL_OK) return KL_ECUDA;
     return prof_mark(ev1, s);
   }
@@ -377,8 +385,12 @@ int launch_render(const kl_params* p, const Plan& L, const View& V, const Tables
   // warp-sized items (32 prefixes), about 12 per resident warp
   const Work Wk = make_work(L, 32, L.npairs, sms * occ * (BT / 32), p->chunk_pairs);
   if (prof_mark(ev0, s) != KL_OK) return KL_ECUDA;
-  if (launch_dependent(words_kernel<BT>(p->precision), dim3(sms * occ), dim3(BT), s, T, L, V, Wk,
-                       img, cnt) != KL_OK)
+  // (a mixed render's queue also holds the fallback items, whose number only the
+  // device knows)
+  const dim3 grid =
+      p->precision == KL_MIXED ? dim3(sms * occ) : words_grid(Wk, sms * occ, BT);
+  if (launch_dependent(words_kernel<BT>(p->precision), grid, dim3(BT), s, T, L, V, Wk, img,
+                       cnt) != KL_OK)
     return KL_ECUDA;
   return prof_mark(ev1, s);
 }

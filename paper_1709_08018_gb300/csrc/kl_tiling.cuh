@@ -178,15 +178,16 @@ __global__ void __launch_bounds__(BT, 1024 / BT) tiling_words_kernel(
     unsigned long long* counters) {
   __shared__ WarpQueue s_queue[BT / 32];
   __shared__ ExactCtx s_ctx[BT / 32];
+  __shared__ unsigned long long s_counts[KL_N_COUNTERS];
   const uint32_t wi = threadIdx.x >> 5, lane = threadIdx.x & 31;
   ExactCtx& C = s_ctx[wi];
+  block_counts_begin(s_counts);
   pdl_wait();
   WordWarp<PREC> w(&C, &s_queue[wi]);
   const uint32_t roots = short_roots(S.k0), first = S.items[0], total = S.items[S.n];
   uint32_t cur = kMaxLengths;  // the length whose context the warp holds
-  for (;;) {
-    const uint32_t item = next_item_warp(S.T[0].fbcount + 1);
-    if (item >= total) break;
+  for (uint32_t item = first_item_warp(); item < total;
+       item = later_item_warp(S.T[0].fbcount + 1, total)) {
     if (item < first) {
       const uint32_t r = item * 32u + lane;
       UnitTally t = {0u, 0u, 0u};
@@ -210,7 +211,8 @@ __global__ void __launch_bounds__(BT, 1024 / BT) tiling_words_kernel(
     word_item(w, item - S.items[i], S.Wk[i], S.L[i], V, C.T, img);
   }
   if (cur < kMaxLengths) w.drain(1);
-  w.finish(counters);
+  w.finish(s_counts);
+  block_counts_end(s_counts, counters);
 }
 
 // ---------------------------------------------------------------------------
