@@ -53,7 +53,8 @@ constexpr uint32_t kNear32 = 128u;   // words on the FP64 map, with an FP32 reco
 enum WordTables : int {
   kPlainTables,   // FP32 records of the prefixes on the FP32 map
   kFilterTables,  // filter constants (kl_filter.cuh)
-  kCullTables     // FP32 records of all prefixes in range (kl_cull.cuh)
+  kCullTables,    // FP32 records of all prefixes in range (kl_cull.cuh)
+  kSizeTables     // and the prefixes' size classes (single culled renders)
 };
 
 // FP64 fallback work unit: a chunk of this many suffix points.
@@ -642,6 +643,27 @@ __device__ __forceinline__ void prefix_rec(const View& V, const Plan& L, double 
   R.fl = fl;
 }
 
+// Size classes of a single culled render (kl_cull.cuh): a prefix's image of a
+// fixed disk scales with |beta|, so its class is the exponent of the larger part
+// of sx beta, the largest sizes first (direct-form prefixes, all of whose words
+// are evaluated, before them).  The ordered slots and the classes' counts and
+// fill levels (4 x 32 each) lie in the fallback list's place, which culled renders
+// do not use.  Plans of fewer than kMinSizeSlots slots keep the slot order: placing
+// them costs 7 us (length 14, 324 slots, 1000 x 507: 81 against 74 us); from 8,748
+// on (length 18) it pays.
+constexpr uint32_t kMinSizeSlots = 8192;
+__device__ __forceinline__ uint32_t size_class(const Pre64& c, uint32_t flags) {
+  if (flags & kDirect) return 0u;
+  const int e = (int)(max(abs_hi(c.c1), abs_hi(c.c2)) >> 20) - 1023;
+  return (uint32_t)min(max(20 - e, 0), 31);
+}
+__device__ __forceinline__ uint32_t* size_order(const Tables& T) {
+  return reinterpret_cast<uint32_t*>(T.fb);
+}
+__device__ __forceinline__ uint32_t* size_counts(const Plan& L, const Tables& T) {
+  return size_order(T) + 4ull * L.np;
+}
+
 // Suffix slot `slot` of the combine pass: the suffix point in the formats that
 // the words of precision prec read.
 __device__ __forceinline__ void suffix_entry(const Plan& L, int prec, uint32_t slot,
@@ -718,10 +740,11 @@ __device__ void combine_entry(const View& V, const Plan& L, double ptol, int pre
     else
       R.fl |= kNoFilter;
   } else {
-    if (what == kCullTables && !(R.fl & (kOnFp32 | kDirect | kWide))) R.fl |= kNear32;
+    if (what >= kCullTables && !(R.fl & (kOnFp32 | kDirect | kWide))) R.fl |= kNear32;
     if (R.fl & (kOnFp32 | kNear32)) T.pre32[slot] = pre32_of(R.c64);
   }
   T.flags[slot] = R.fl;
+  if (what == kSizeTables) atomicAdd(size_counts(L, T) + 32 * x + size_class(R.c64, R.fl), 1u);
 }
 
 // ---------------------------------------------------------------------------

@@ -23,13 +23,15 @@ constexpr uint32_t kPartLanes = 8;
 // parts skipped) when the prefix tables are already in place, whose fallback
 // count is then kept.
 __global__ void parts_kernel(Group G, Plan L, int renorm, Tables T, Clear C,
-                             uint32_t part_blocks, uint32_t first) {
+                             uint32_t part_blocks, uint32_t first, int sized) {
   pdl_trigger();
   if (blockIdx.x < part_blocks) {
     if (blockIdx.x == 0) {
       if (threadIdx.x == 0 && first == 0) T.fbcount[0] = 0u;  // fallback prefixes
       if (threadIdx.x == 1) T.fbcount[1] = 0u;                // the work queue
       if (C.counters && threadIdx.x < KL_N_COUNTERS) C.counters[threadIdx.x] = 0ull;
+      if (sized)
+        for (uint32_t i = threadIdx.x; i < 256u; i += blockDim.x) size_counts(L, T)[i] = 0u;
     }
     // kPartLanes entries per block: each entry is one long chain of dependent
     // FP64 operations, so spreading the entries over more SMs shortens the
@@ -126,11 +128,11 @@ __global__ void __launch_bounds__(BT, 1024 / BT) render_words_kernel(
 // culled renders (kl_params.cull; the culling itself is in kl_cull.cuh)
 
 // Disks of all culling blocks, then the prefix norms (cull_disk_unit).
-__global__ void __launch_bounds__(128) disk_kernel(Plan L, Tables T) {
+__global__ void __launch_bounds__(128) disk_kernel(Plan L, Tables T, bool sized) {
   pdl_trigger();
   pdl_wait();
   const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (warp < cull_disk_units(L)) cull_disk_unit(L, T, warp, threadIdx.x & 31);
+  if (warp < cull_disk_units(L)) cull_disk_unit(L, T, warp, threadIdx.x & 31, sized);
 }
 
 // Culled render of one group: persistent warps take items of 32 prefixes x
@@ -138,7 +140,7 @@ __global__ void __launch_bounds__(128) disk_kernel(Plan L, Tables T) {
 template <int BT, bool MIXED>
 __global__ void __launch_bounds__(BT, 1024 / BT) cull_kernel(
     Tables T, Plan L, View V, Work Wk, uint32_t* __restrict__ img,
-    unsigned long long* counters) {
+    unsigned long long* counters, bool sized) {
   __shared__ unsigned long long s_stack[BT / 32][kCullStack];
   __shared__ unsigned long long s_leaf[BT / 32][kLeafQueue];
   __shared__ CullLevels C;
@@ -154,7 +156,7 @@ __global__ void __launch_bounds__(BT, 1024 / BT) cull_kernel(
   for (;;) {
     const uint32_t item = next_item_warp(T.fbcount + 1);
     if (item >= Wk.n_items) break;
-    cull_item(w, item, Wk, L, V, T, img, top_blocks);
+    cull_item(w, item, Wk, L, V, T, img, top_blocks, sized);
   }
   w.finish(L, V, T, img);
   w.t.flush(img);
@@ -292,7 +294,8 @@ int build_tables(const kl_params* p, const Plan& L, const View& V, const Group& 
   const int sms = sm_count();
   if (sms <= 0) return KL_ECUDA;
   parts_kernel<<<part_blocks + clear_blocks(C, sms), 32, 0, st>>>(G, L, (int)p->renorm_every, T, C,
-                                                          part_blocks, first_part);
+                                                          part_blocks, first_part,
+                                                          what == kSizeTables);
   if (check_launch() != KL_OK) return KL_ECUDA;
   const uint32_t n = combine_count(L) - first_comb;
   return launch_dependent(combine_kernel, dim3(n > 0 ? (n + 127) / 128 : 1u), dim3(128), st, V,
@@ -348,6 +351,11 @@ WordsKernel words_kernel(uint32_t precision) {
   }
 }
 
+// What the combine pass of a culled render of plan L prepares.
+WordTables cull_tables(const Plan& L) {
+  return 4u * L.np >= kMinSizeSlots ? kSizeTables : kCullTables;
+}
+
 // Persistent blocks for the items of Wk: the resident ones, or fewer where not
 // every warp of them would get an item.
 dim3 words_grid(const Work& Wk, int slots, int bt) {
@@ -363,7 +371,8 @@ int launch_render(const kl_params* p, const Plan& L, const View& V, const Tables
   if (p->cull) {
     // block disks (a programmatic dependent of combine), then the culled render
     const uint32_t warps = cull_disk_units(L);
-    if (launch_dependent(disk_kernel, dim3((warps + 3u) / 4u), dim3(128), s, L, T) != KL_OK)
+    const bool sized = cull_tables(L) == kSizeTables;
+    if (launch_dependent(disk_kernel, dim3((warps + 3u) / 4u), dim3(128), s, L, T, sized) != KL_OK)
       return KL_ECUDA;
     const bool mixed = p->precision == KL_MIXED;
     const void* k = mixed ? (const void*)cull_kernel<BT, true> : (const void*)cull_kernel<BT, false>;
@@ -374,9 +383,9 @@ int launch_render(const kl_params* p, const Plan& L, const View& V, const Tables
     if (prof_mark(ev0, s) != KL_OK) return KL_ECUDA;
     const dim3 grid = words_grid(Wk, sms * occ, BT);
     const int st = mixed ? launch_dependent(cull_kernel<BT, true>, grid, dim3(BT), s, T, L, V, Wk,
-                                            img, cnt)
+                                            img, cnt, sized)
                          : launch_dependent(cull_kernel<BT, false>, grid, dim3(BT), s, T, L, V,
-                                            Wk, img, cnt);
+                                            Wk, img, cnt, sized);
     if (st != KL_OK) return KL_ECUDA;
     return prof_mark(ev1, s);
   }
@@ -479,7 +488,7 @@ int render_length(const kl_params* p, uint32_t* d_image, unsigned long long* cnt
   Clear C{};
   if (!p->accumulate) C = {d_image, (size_t)p->width * p->height, cnt};
   st = build_tables(p, L, V, G, T, s, C, prev && prefix_tables_shared(*prev, L, p),
-                    p->cull                       ? kCullTables
+                    p->cull                       ? cull_tables(L)
                     : p->precision == KL_MIXED ? kPlainTables
                                                : kFilterTables);
   if (st != KL_OK) return st;
