@@ -46,12 +46,12 @@ constexpr uint32_t kFallback = 8u;   // KL_MIXED, KL_DF64: words of this prefix 
 constexpr uint32_t kDfRange = 16u;   // a pole-form constant outside the double-float range
 constexpr uint32_t kNoFilter = 32u;  // no filter constants: words take the exact map (kl_filter.cuh)
 constexpr uint32_t kOnFp32 = 64u;    // KL_MIXED: words on the FP32 map (its record is pre32's)
-constexpr uint32_t kNear32 = 128u;   // words on the FP64 map, with an FP32 record for the certified
-                                     // tests of a culled render
+constexpr uint32_t kNear32 = 128u;   // words on the FP64 map, with an FP32 record for certified
+                                     // tests (culled and mixed renders)
 
 // What the words of a render read beside the FP64 records (combine_entry).
 enum WordTables : int {
-  kPlainTables,   // FP32 records of the prefixes on the FP32 map
+  kPlainTables,   // FP32 records of the prefixes on the FP32 map; KL_MIXED: of all in range
   kFilterTables,  // filter constants (kl_filter.cuh)
   kCullTables,    // FP32 records of all prefixes in range (kl_cull.cuh)
   kSizeTables     // and the prefixes' size classes (single culled renders)
@@ -740,7 +740,7 @@ __device__ void combine_entry(const View& V, const Plan& L, double ptol, int pre
     else
       R.fl |= kNoFilter;
   } else {
-    if (what >= kCullTables && !(R.fl & (kOnFp32 | kDirect | kWide))) R.fl |= kNear32;
+    if ((what >= kCullTables || prec == KL_MIXED) && !(R.fl & (kOnFp32 | kDirect | kWide))) R.fl |= kNear32;
     if (R.fl & (kOnFp32 | kNear32)) T.pre32[slot] = pre32_of(R.c64);
   }
   T.flags[slot] = R.fl;
@@ -958,13 +958,58 @@ __device__ __forceinline__ void words64(const Pre64& k, bool direct, const doubl
   if (BBOX) box_merge(*B, slot, c0, c1, r0, r1);
 }
 
+// FP64 words of a pole-form prefix on suffix points [j0, j1): each in FP32 first
+// (k: the prefix's constants rounded to FP32), in FP64 where the bound does not
+// settle the pixel, so every word lands where FP64 puts it.  Error, R = |M| / |w|
+// an upper bound on both parts of the offset from alpha, q = (|v| + |gamma|) /
+// |w|: the rounded sum w is off by eps (1 + q) |w|, which moves the offset by at
+// most twice that of R; rounding M, the products, |w|^2, its reciprocal root and
+// the last products, 18 eps R; the sum with alpha, eps of its parts.  Below eps R
+// (22 + 2 q) in all; the code takes eps R (64 + 8 q), and settles nothing where
+// 8 eps q >= 1/4.
+__device__ __forceinline__ void near_words64(const Pre32& k, const Pre64* __restrict__ c64,
+                                             float nrm, const float4* s32, const double2* s64,
+                                             uint32_t j0, uint32_t j1, const View& V, Tally& t,
+                                             uint32_t* __restrict__ img) {
+  const float c0 = 4.0f * kEps24 * (2.0f + fabsf(k.axf) + fabsf(k.ayf));
+  const float ag = fabsf(k.gr) + fabsf(k.gi), magic = 12582912.0f;
+  for (uint32_t j = j0; j < j1; ++j) {
+    const float4 s = __ldg(s32 + j / 2u);
+    const float vr = j & 1u ? s.y : s.x, vi = j & 1u ? s.w : s.z;
+    const float wr = vr + k.gr, wi = vi + k.gi;
+    const float m = fmaf(wr, wr, wi * wi), rw = rsqrtf(m), r = rw * rw;
+    const float X = fmaf(k.c1, wr, k.c2 * wi) * r, Y = fmaf(k.c3, wr, k.c4 * wi) * r;
+    const float q = 8.0f * kEps24 * (ag + fabsf(vr) + fabsf(vi)) * rw;
+    const float E = fmaf(nrm * rw, q + 64.0f * kEps24, c0);
+    const float u = X + k.axf, v = Y + k.ayf;
+    const int ul = __float_as_int(__fadd_rd(u - E, magic));
+    const int uh = __float_as_int(__fadd_rd(u + E, magic));
+    const int vl = __float_as_int(__fadd_rd(v - E, magic));
+    const int vh = __float_as_int(__fadd_rd(v + E, magic));
+    int pix;
+    if (m > 1e-30f && m < 1e30f && q < 0.25f && E < 0.25f && fabsf(u) < 0x1p20f && fabsf(v) < 0x1p20f && ul == uh &&
+        vl == vh) {
+      const int col = ul - k.kx, row = vl - k.ky;
+      pix = ((uint32_t)col < V.W && (uint32_t)row < V.H) ? row * (int)V.W + col : -1;
+    } else {
+      const double2 z = __ldg(s64 + j);
+      double uu, vv;
+      uv_pole64(*c64, z.x, z.y, uu, vv);
+      pix = pixel64(uu, vv, V);
+    }
+    t.add(pix, img);
+  }
+}
+
 // Mixed-mode FP64 fallback unit (kept out of line so that its registers do
 // not bind the FP32 loop): (fallback prefix, one of its three suffix letters,
 // a chunk of kFbChunk suffix points).  Chunks past the end are empty.
 template <bool BBOX = false>
 __device__ __noinline__ UnitTally fallback_unit(const Pre64* __restrict__ pre,
                                                 const uint32_t* __restrict__ flags,
-                                                const double2* __restrict__ suf, uint32_t slot,
+                                                const double2* __restrict__ suf,
+                                                const Pre32* __restrict__ pre32,
+                                                const float4* __restrict__ suf32, uint32_t slot,
                                                 uint32_t k, uint32_t c, uint32_t np, uint32_t ns,
                                                 View V, uint32_t* __restrict__ img,
                                                 BoxRef B = BoxRef{}) {
@@ -974,8 +1019,18 @@ __device__ __noinline__ UnitTally fallback_unit(const Pre64* __restrict__ pre,
   if (j0 >= ns) return {0u, 0u, 0u};
   const uint32_t j1 = min(ns, j0 + kFbChunk);
   Tally t;
-  words64<BBOX>(pre[slot], flags[slot] & kDirect, suf + (size_t)u * ns, j0, j1, V, t, img, &B,
-                slot);
+  const uint32_t fl = flags[slot];
+  if (!BBOX && (fl & kNear32)) {
+    const Pre32 k32 = pre32[slot];
+    // the Frobenius norm bounds the operator norm
+    const float nrm = sqrtf(fmaf(k32.c1, k32.c1, k32.c2 * k32.c2) +
+                            fmaf(k32.c3, k32.c3, k32.c4 * k32.c4)) * (1.0f + 0x1p-16f);
+    near_words64(k32, pre + slot, nrm, suf32 + (size_t)u * ((ns + 1u) / 2u),
+                 suf + (size_t)u * ns, j0, j1, V, t, img);
+    t.flush(img);
+  } else {
+    words64<BBOX>(pre[slot], fl & kDirect, suf + (size_t)u * ns, j0, j1, V, t, img, &B, slot);
+  }
   return {j1 - j0, t.in_window, t.atomics};
 }
 

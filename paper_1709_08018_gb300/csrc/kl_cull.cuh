@@ -159,49 +159,6 @@ __device__ __forceinline__ void mixed_block_words(uint32_t slot, int u, uint32_t
   if (j1 > j0) mixed_slot_words(slot, u, j0 / 2u, j1 / 2u, L, V, T, t, words, img);
 }
 
-// FP64 words of a pole-form prefix on suffix points [j0, j1): each in FP32 first
-// (k: the prefix's constants rounded to FP32), in FP64 where the bound does not
-// settle the pixel, so every word lands where FP64 puts it.  Error, R = |M| / |w|
-// an upper bound on both parts of the offset from alpha, q = (|v| + |gamma|) /
-// |w|: the rounded sum w is off by eps (1 + q) |w|, which moves the offset by at
-// most twice that of R; rounding M, the products, |w|^2, its reciprocal root and
-// the last products, 18 eps R; the sum with alpha, eps of its parts.  Below eps R
-// (22 + 2 q) in all; the code takes eps R (64 + 8 q), and settles nothing where
-// 8 eps q >= 1/4.
-__device__ __forceinline__ void near_words64(const Pre32& k, const Pre64* __restrict__ c64,
-                                             float nrm, const float4* s32, const double2* s64,
-                                             uint32_t j0, uint32_t j1, const View& V, Tally& t,
-                                             uint32_t* __restrict__ img) {
-  const float c0 = 4.0f * kEps24 * (2.0f + fabsf(k.axf) + fabsf(k.ayf));
-  const float ag = fabsf(k.gr) + fabsf(k.gi), magic = 12582912.0f;
-  for (uint32_t j = j0; j < j1; ++j) {
-    const float4 s = __ldg(s32 + j / 2u);
-    const float vr = j & 1u ? s.y : s.x, vi = j & 1u ? s.w : s.z;
-    const float wr = vr + k.gr, wi = vi + k.gi;
-    const float m = fmaf(wr, wr, wi * wi), rw = rsqrtf(m), r = rw * rw;
-    const float X = fmaf(k.c1, wr, k.c2 * wi) * r, Y = fmaf(k.c3, wr, k.c4 * wi) * r;
-    const float q = 8.0f * kEps24 * (ag + fabsf(vr) + fabsf(vi)) * rw;
-    const float E = fmaf(nrm * rw, q + 64.0f * kEps24, c0);
-    const float u = X + k.axf, v = Y + k.ayf;
-    const int ul = __float_as_int(__fadd_rd(u - E, magic));
-    const int uh = __float_as_int(__fadd_rd(u + E, magic));
-    const int vl = __float_as_int(__fadd_rd(v - E, magic));
-    const int vh = __float_as_int(__fadd_rd(v + E, magic));
-    int pix;
-    if (m > 1e-30f && m < 1e30f && q < 0.25f && E < 0.25f && fabsf(u) < 0x1p20f && fabsf(v) < 0x1p20f && ul == uh &&
-        vl == vh) {
-      const int col = ul - k.kx, row = vl - k.ky;
-      pix = ((uint32_t)col < V.W && (uint32_t)row < V.H) ? row * (int)V.W + col : -1;
-    } else {
-      const double2 z = __ldg(s64 + j);
-      double uu, vv;
-      uv_pole64(*c64, z.x, z.y, uu, vv);
-      pix = pixel64(uu, vv, V);
-    }
-    t.add(pix, img);
-  }
-}
-
 // Disk of culling block `disk` of plan L (all lanes of a warp take part),
 // from the FP32 points that the mixed per-word path reads: center = middle of
 // their bounding box, radius = largest distance from it, with a relative

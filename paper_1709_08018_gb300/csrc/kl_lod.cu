@@ -155,8 +155,8 @@ __global__ void __launch_bounds__(BT, 1536 / BT) lod_exact_kernel(
       if (MIXED && unit < fb_units) {
         const uint32_t e = unit / (3u * chunks), rem = unit % (3u * chunks);
         const uint32_t slot = (uint32_t)(T.fb[e] & 0xFFFFFFFFull);
-        const UnitTally r = fallback_unit<true>(T.pre64, T.flags, T.suf64, slot, rem / chunks,
-                                                rem % chunks, L.np, L.ns, V, img, B);
+        const UnitTally r = fallback_unit<true>(T.pre64, T.flags, T.suf64, T.pre32, T.suf32p,
+                                                slot, rem / chunks, rem % chunks, L.np, L.ns, V, img, B);
         words += r.words;
         fp64_words += r.words;
         t.in_window += r.in_window;
