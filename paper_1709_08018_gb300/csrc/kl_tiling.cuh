@@ -39,10 +39,13 @@ __device__ __forceinline__ dc short_map(const Group& G, int x, dc z) {
   return {(num.re * den.re + num.im * den.im) * rc, (num.im * den.re - num.re * den.im) * rc};
 }
 
-// Roots of the walk: the words of lengths 1 .. max(k0 - kShortWalk, 1); those
-// of the largest length are walked, the others stand for themselves.
+// Roots of the walk: the words of lengths 1 .. short_root_length; those of the
+// largest length are walked, the others stand for themselves.  Only all kShortTiling
+// lengths have words enough to fill the FP64 pipe; below, the chain of one lane
+// is what takes the time, and every word is a root (7 letters, 700 x 500: 23 us,
+// walked 26).
 __host__ __device__ __forceinline__ uint32_t short_root_length(uint32_t k0) {
-  return k0 > (uint32_t)kShortWalk ? k0 - (uint32_t)kShortWalk : 1u;
+  return k0 >= kShortTiling ? k0 - (uint32_t)kShortWalk : k0;
 }
 __host__ __device__ __forceinline__ uint32_t short_roots(uint32_t k0) {
   uint32_t total = 0, nk = 4;
