@@ -41,7 +41,8 @@ struct FsaDev {
   unsigned long long ways[kFsaMaxDepth + 1][kFsaStates];
 };
 
-// One generator in FP32 with the 1-norms of its entries (the leaf test).
+// One generator in FP32 with the 1-norms of its entries, nq and ns with kTiny
+// (the leaf test).
 struct FsaMap32 {
   float v[8];           // p, q, r, s (re, im)
   float np, nq, nr, ns;
@@ -84,14 +85,22 @@ __device__ __forceinline__ dc fsa_map(const double* M, dc z) {
 // is off by less than 12 eps (A + |w| B) / |den| plus 13 eps |w| for its own
 // roundings and the reciprocal root, and the pixel transform adds 5 eps of
 // |w| + |x0| (|y1|); the code takes 20 eps for the last two.
+// Range: a map does not change with the scale of its matrix, so entries of any
+// size are legal.  |den|^2 outside (1e-30, 1e30) or |z| from 1e15 on settles
+// nothing: past 1.8e19 |den|^2 overflows and the quotient and its bound would
+// both be 0.  Within, what FP32 loses to underflow, 2^-150 times |z| < 2^50 in an
+// entry and 2^-149 / |den|, |den| > 2^-50, in a product of the quotient, is below
+// kTiny in A and B times 12 eps.
+constexpr float kTiny = 0x1p-76f;
 constexpr int kUnsettled = -2;
 __device__ __forceinline__ int fsa_leaf32(const FsaMap32& M, float zr, float zi, const View& V,
                                           float x0, float y1, float sx, float sy) {
   const float* v = M.v;
   const float nr = fmaf(v[0], zr, fmaf(-v[1], zi, v[2])), ni = fmaf(v[0], zi, fmaf(v[1], zr, v[3]));
   const float dr = fmaf(v[4], zr, fmaf(-v[5], zi, v[6])), di = fmaf(v[4], zi, fmaf(v[5], zr, v[7]));
+  const float m = fmaf(dr, dr, di * di);
   float rd;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rd) : "f"(fmaf(dr, dr, di * di)));
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rd) : "f"(m));
   const float rc = rd * rd;
   const float wr = fmaf(nr, dr, ni * di) * rc, wi = fmaf(ni, dr, -(nr * di)) * rc;
   const float az = fabsf(zr) + fabsf(zi), aw = fabsf(wr) + fabsf(wi);
@@ -100,7 +109,9 @@ __device__ __forceinline__ int fsa_leaf32(const FsaMap32& M, float zr, float zi,
   const float e = fmaf(12.0f * 0x1p-24f * rd, fmaf(aw, B, A), 20.0f * 0x1p-24f * aw);
   const float eu = fmaf(5.0f * 0x1p-24f, fabsf(x0), e) * sx;
   const float ew = fmaf(5.0f * 0x1p-24f, fabsf(y1), e) * sy;
-  if (!(12.0f * 0x1p-24f * B * rd < 0.25f && eu < 0.25f && ew < 0.25f)) return kUnsettled;
+  if (!(m > 1e-30f && m < 1e30f && az < 1e15f && 12.0f * 0x1p-24f * B * rd < 0.25f &&
+        eu < 0.25f && ew < 0.25f))
+    return kUnsettled;
   const float W = (float)V.W, H = (float)V.H;
   if (u < -eu || u > W + eu || w < -ew || w > H + ew) return -1;
   const int c0 = (int)floorf(u - eu), c1 = (int)floorf(u + eu);
@@ -212,9 +223,9 @@ __global__ void __launch_bounds__(kFsaThreads) fsa_render_kernel(
   if (threadIdx.x < m) {
     FsaMap32& f = S.f[threadIdx.x];
     f.np = fabsf(f.v[0]) + fabsf(f.v[1]);
-    f.nq = fabsf(f.v[2]) + fabsf(f.v[3]);
+    f.nq = fabsf(f.v[2]) + fabsf(f.v[3]) + kTiny;
     f.nr = fabsf(f.v[4]) + fabsf(f.v[5]);
-    f.ns = fabsf(f.v[6]) + fabsf(f.v[7]);
+    f.ns = fabsf(f.v[6]) + fabsf(f.v[7]) + kTiny;
   }
   __syncthreads();
   FsaWalk w = {&S, &queues[threadIdx.x / 32], V, (float)V.x0, (float)V.y1, (float)V.sx,
