@@ -263,6 +263,10 @@ inline Work make_work(const Plan& L, int bt, uint32_t units, int slots, uint32_t
     W.chunk = chunk_units < units ? chunk_units : units;
   }
   if (W.chunk < 1) W.chunk = 1;
+  // at most 2^31 items (the queue counts in 32 bits): the longest words in the
+  // smallest chunks would need 5.9e9
+  const uint32_t least = (uint32_t)((units * base + (1ull << 31) - 1) >> 31);
+  if (W.chunk < least) W.chunk = least;
   W.n_chunks = (units + W.chunk - 1) / W.chunk;
   W.n_items = (uint32_t)(base * W.n_chunks);
   return W;
