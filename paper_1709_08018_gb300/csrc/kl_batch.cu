@@ -418,7 +418,7 @@ extern "C" int kl_batch_create(const kl_params* params, uint32_t n_groups, kl_ba
     return KL_ECUDA;
   }
   const uint32_t chunk = p0.chunk_pairs ? p0.chunk_pairs : 64u;
-  uint64_t parts = 0, comb = 0, items = 0, fb = 0, disk = 0;
+  uint64_t parts = 0, comb = 0, fb = 0, disk = 0;
   size_t off = 0;
   b->off_desc = off; off = align256(off + n_groups * sizeof(GroupDesc));
   b->off_bases = off; off = align256(off + b->bases.size() * sizeof(uint32_t));
@@ -429,21 +429,32 @@ extern "C" int kl_batch_create(const kl_params* params, uint32_t n_groups, kl_ba
       delete b;
       return st;
     }
-    // culled: warp items of 32 prefixes x one top-level block
-    b->works[g] = b->cull ? make_work(L, 32, L.cnb[L.clev - 1], 1, 1u)
-                          : make_work(L, 32, L.npairs, 1, chunk);
     b->bases[g] = (uint32_t)parts;
     b->bases[(n_groups + 1) + g] = (uint32_t)comb;
-    b->bases[2 * (n_groups + 1) + g] = (uint32_t)items;
     b->bases[3 * (n_groups + 1) + g] = (uint32_t)disk;
     parts += parts_count(L);
     comb += combine_count(L);
-    items += b->works[g].n_items;
     if (b->cull) disk += cull_disk_units(L);
     fb += 4ull * L.np;
     const uint32_t cg = (L.ns + kFbChunk - 1) / kFbChunk;
     if (cg > b->cmax) b->cmax = cg;
   }
+  // the groups' items with chunks of c pairs (culled: of one top-level block)
+  auto make_items = [&](uint32_t c) {
+    uint64_t items = 0;
+    for (uint32_t g = 0; g < n_groups; ++g) {
+      const Plan& L = b->plans[g];
+      b->works[g] = b->cull ? make_work(L, 32, L.cnb[L.clev - 1], 1, 1u)
+                            : make_work(L, 32, L.npairs, 1, c);
+      b->bases[2 * (n_groups + 1) + g] = (uint32_t)items;
+      items += b->works[g].n_items;
+    }
+    return items;
+  };
+  uint64_t items = make_items(chunk);
+  // FP64 batches that fitted with a block's prefixes to an item still fit
+  if (items >= (1ull << 31) && !b->mixed && !b->cull)
+    items = make_items((chunk < (1u << 20) ? chunk : 1u << 20) * (uint32_t)(b->bt / 32));
   if (parts >= (1ull << 32) || comb >= (1ull << 32) || items >= (1ull << 31) ||
       disk >= (1ull << 31) || 3ull * b->cmax * fb >= (1ull << 32)) {
     delete b;

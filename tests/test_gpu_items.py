@@ -26,3 +26,20 @@ def test_longest_words_in_the_smallest_chunks(kl, prec):
     image, counters = kl.render(p)
     assert int(counters[0]) + int(counters[1]) == kl.word_count(24)
     assert int(image.long().bitwise_and(0xFFFFFFFF).sum()) % 2 ** 32 == int(counters[0]) % 2 ** 32
+
+
+def test_batch_of_long_words_in_the_smallest_chunks(kl):
+    """Four FP64 groups of 22 letters, one pair of points to a chunk: 2.6e9
+    items of 32 prefixes, 6.5e8 with chunks four times as long."""
+    make = lambda side: kl.params_init(2.1 + 0.01j, 2.3, 22, side, side, (-1.5, 1.5, -1.5, 1.5),
+                                       kl.FP64, chunk_pairs=1)
+    images, counters = kl.Batch([make(64)] * 4).render()
+    want, count = kl.render(make(64))
+    for g in range(4):
+        assert int(counters[g, 0]) + int(counters[g, 1]) == kl.word_count(22)
+        assert int(images[g].long().sum()) == int(counters[g, 0])
+    assert bool((images[1:] == images[0]).all())
+    # the batch splits the words at other letters: words on a pixel's edge may
+    # lie on either side of it
+    assert abs(int(counters[0, 0]) - int(count[0])) <= 1000
+    assert int((images[0] - want).abs().sum()) <= 1e-6 * kl.word_count(22)
