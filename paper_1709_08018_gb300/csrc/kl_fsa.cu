@@ -19,10 +19,16 @@
 // + 1/2 FP64 maps per kept string of the once-punctured torus: a leaf needs
 // only its pixel, so its own map is made in FP32 with an error bound, and in
 // FP64 (the same operations as for any node) when the bound does not settle
-// the pixel (a few leaves in 100; they wait in a queue until a warp has 32).  h = 4: roots enough to fill the
-// GPU from length 13 on; h = 3 leaves 1.4 times the FP64 maps (13 letters at
-// 2000 x 1500: 109 against 96 us, and 1624 us for the scan; the FP64 pipe's
-// share is 46 us).
+// the pixel (a few leaves in 100; they wait in a queue until a warp has 32).
+//
+// Height.  One lane walks a subtree alone, so h is the largest up to 4 that
+// leaves every SM three warps of roots.  Measured at 1500 x 1100, h = 0 .. 4, torus
+// table: 12 letters 386, 139, 71, 49 and 81 us (26,244 roots at h = 3, 8,748 at
+// 4), 13 letters 1198, 394, 176, 112 and 96 us, 9 letters 25, 24, 26, 39 and 78;
+// nine letters, every string kept: 5 letters 31, 23, 50, 305 and 2567 us, 7 letters
+// 1445, 174, 123, 309 and 2644; six: 8 letters 593, 117, 82, 118 and 620.  (13 letters
+// at 2000 x 1500, torus: scanning all strings took 1624 us; the FP64 pipe's
+// share of the 96 is 46.)
 #include "kl_common.cuh"
 
 namespace {
@@ -31,6 +37,7 @@ constexpr int kFsaThreads = 64;
 constexpr int kFsaMaxDepth = 32;
 constexpr int kFsaStates = KL_FSA_MAX_LETTERS + 1;
 constexpr int kFsaSubtree = 4;  // letters walked below a root, at most
+constexpr uint32_t kFsaRootsPerSm = 96;
 
 struct FsaDev {
   uint32_t m, d;
@@ -338,11 +345,13 @@ extern "C" int kl_render_fsa(const kl_fsa* f, const kl_params* p, uint32_t* d_im
   for (uint32_t k = 0; k < 8 * F.m; ++k) F.g[k] = f->gens[k];
   for (uint32_t k = 0; k < 2 * F.m; ++k) F.seed[k] = f->seeds[k];
   fsa_ways(f, F.d, F.ways);
-  const uint32_t h = F.d - 1 < (uint32_t)kFsaSubtree ? F.d - 1 : (uint32_t)kFsaSubtree;
+  int sms = 0, occ = 0;
+  if ((sms = sm_count()) <= 0) return KL_ECUDA;
+  uint32_t h = F.d - 1 < (uint32_t)kFsaSubtree ? F.d - 1 : (uint32_t)kFsaSubtree;
+  while (h > 0 && F.ways[F.d - h][0] < kFsaRootsPerSm * (unsigned long long)sms) --h;
   const FsaKernel kernels[kFsaSubtree + 1] = {fsa_render_kernel<0>, fsa_render_kernel<1>,
                                               fsa_render_kernel<2>, fsa_render_kernel<3>,
                                               fsa_render_kernel<4>};
-  int sms = 0, occ = 0;
   if (device_slots((const void*)kernels[h], kFsaThreads, &sms, &occ) != KL_OK) return KL_ECUDA;
   const unsigned long long roots = F.ways[F.d - h][0];
   const unsigned long long blocks = (roots + kFsaThreads - 1) / kFsaThreads;
