@@ -853,8 +853,8 @@ __device__ __forceinline__ uint32_t next_item_warp(uint32_t* queue) {
 // The items of a persistent launch: every warp's first one by its place in the
 // grid, consecutive items in different blocks, the others from the queue.  A
 // launch with an item or less per warp makes no queue atomic at all.  With the
-// counters added per block (below) and no blocks without items: FP64 gasket,
-// length 10, 27.4 -> 24.6 us; the length-18 render the same.  The mixed and the
+// counters added per block (below): FP64 gasket, length 10, 27.4 -> 24.6 us; the
+// length-18 render the same.  The mixed and the
 // culled renders keep to the queue from the first item on: their first items are
 // the slow ones, which the queue spreads better (0.5% slower otherwise).
 __device__ __forceinline__ uint32_t first_item_warp() {
