@@ -59,6 +59,11 @@ enum WordTables : int {
 
 // FP64 fallback work unit: a chunk of this many suffix points.
 constexpr uint32_t kFbChunk = 64;
+// Twice that where all of a render's prefixes in chunks of 64 points would overflow
+// the 32-bit unit count (24 letters: 12 np ns / 64 = 5.9e9 units).
+__host__ __device__ __forceinline__ uint32_t fb_chunk(uint32_t np, uint32_t ns) {
+  return 12ull * np * ((ns + kFbChunk - 1) / kFbChunk) >> 32 ? 2 * kFbChunk : kFbChunk;
+}
 
 struct Plan {
   int d, p, s;
@@ -1004,7 +1009,7 @@ __device__ __forceinline__ void near_words64(const Pre32& k, const Pre64* __rest
 // Mixed-mode FP64 fallback unit (kept out of line so that its registers do
 // not bind the FP32 loop; FP32 with a bound first: gasket, 14 letters, 1024 x 519,
 // 78 -> 44 us, the fallback words had kept the FP64 pipe busy after the others): (fallback prefix, one of its three suffix letters,
-// a chunk of kFbChunk suffix points).  Chunks past the end are empty.
+// a chunk of fb_chunk suffix points).  Chunks past the end are empty.
 template <bool BBOX = false>
 __device__ __noinline__ UnitTally fallback_unit(const Pre64* __restrict__ pre,
                                                 const uint32_t* __restrict__ flags,
@@ -1016,9 +1021,9 @@ __device__ __noinline__ UnitTally fallback_unit(const Pre64* __restrict__ pre,
                                                 BoxRef B = BoxRef{}) {
   const int x = (int)(slot / np);
   const int u = allowed_letter((int)k, (x + 2) & 3);
-  const uint32_t j0 = c * kFbChunk;
+  const uint32_t len = fb_chunk(np, ns), j0 = c * len;
   if (j0 >= ns) return {0u, 0u, 0u};
-  const uint32_t j1 = min(ns, j0 + kFbChunk);
+  const uint32_t j1 = min(ns, j0 + len);
   Tally t;
   const uint32_t fl = flags[slot];
   if (!BBOX && (fl & kNear32)) {

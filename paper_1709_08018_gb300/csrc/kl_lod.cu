@@ -141,7 +141,7 @@ template <int BT, bool MIXED>
 __global__ void __launch_bounds__(BT, 1536 / BT) lod_exact_kernel(
     Tables T, Plan L, View V, Work Wk, BoxRef B, uint32_t* __restrict__ img,
     unsigned long long* counters) {
-  const uint32_t chunks = (L.ns + kFbChunk - 1) / kFbChunk;
+  const uint32_t len = fb_chunk(L.np, L.ns), chunks = (L.ns + len - 1) / len;
   const uint32_t fb_units = MIXED ? 3u * chunks * (*T.fbcount) : 0u;
   const uint32_t n64 = (fb_units + BT - 1) / BT;
   const uint32_t total = n64 + Wk.n_items;

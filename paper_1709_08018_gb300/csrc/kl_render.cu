@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(BT, 1280 / BT) render_mixed_kernel(
     Tables T, Plan L, View V, Work Wk, uint32_t* __restrict__ img,
     unsigned long long* counters) {
   pdl_wait();
-  const uint32_t chunks = (L.ns + kFbChunk - 1) / kFbChunk;
+  const uint32_t len = fb_chunk(L.np, L.ns), chunks = (L.ns + len - 1) / len;
   const uint32_t fb_units = 3u * chunks * (*T.fbcount);
   const uint32_t n64 = (fb_units + 31) / 32;
   const uint32_t total = n64 + Wk.n_items;

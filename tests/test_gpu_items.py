@@ -43,3 +43,12 @@ def test_batch_of_long_words_in_the_smallest_chunks(kl):
     # lie on either side of it
     assert abs(int(counters[0, 0]) - int(count[0])) <= 1000
     assert int((images[0] - want).abs().sum()) <= 1e-6 * kl.word_count(22)
+
+
+def test_longest_words_on_the_fp64_path(kl):
+    """24 letters, mixed, every prefix far from the window (FP64 words): 5.9e9
+    fallback units of 64 points would overflow the 32-bit unit count."""
+    p = kl.params_init(2.1 + 0.01j, 2.3, 24, 64, 64, (1e9, 1e9 + 1.0, 0.0, 1.0), kl.MIXED)
+    image, counters = kl.render(p)
+    assert int(counters[2]) == int(counters[1]) == kl.word_count(24)
+    assert int(counters[0]) == 0 and not bool(image.any())
