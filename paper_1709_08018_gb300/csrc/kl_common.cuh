@@ -285,6 +285,25 @@ __device__ __forceinline__ void uv_direct64(const Pre64& c, double vr, double vi
   v = __dmul_rn(__dsub_rn(V.y1, zi), V.sy);
 }
 
+// Map M (p, q, r, s as re, im) of the point z with a refined reciprocal instead of
+// divisions, its multiply-adds spelled out so that a value has the same bits wherever
+// the compiler inlines it (the scan's strings and a tiling render's short words).
+__device__ __forceinline__ double mul_sub(double a, double b, double c, double d) {
+  return __fma_rn(a, b, -__dmul_rn(c, d));
+}
+__device__ __forceinline__ double mul_add(double a, double b, double c, double d) {
+  return __fma_rn(a, b, __dmul_rn(c, d));
+}
+__device__ __forceinline__ dc point_map(const double* M, dc z) {
+  const dc num = {__dadd_rn(mul_sub(M[0], z.re, M[1], z.im), M[2]),
+                  __dadd_rn(mul_add(M[0], z.im, M[1], z.re), M[3])};
+  const dc den = {__dadd_rn(mul_sub(M[4], z.re, M[5], z.im), M[6]),
+                  __dadd_rn(mul_add(M[4], z.im, M[5], z.re), M[7])};
+  const double r = rcp64(mul_add(den.re, den.re, den.im, den.im));
+  return {__dmul_rn(mul_add(num.re, den.re, num.im, den.im), r),
+          __dmul_rn(mul_sub(num.im, den.re, num.re, den.im), r)};
+}
+
 // Scalar form of the mixed per-word map (the evaluation kernel); the render
 // evaluates the same operations two words at a time.
 __device__ __forceinline__ void uv_pole32(const Pre32& c, float vr, float vi, float& uf,

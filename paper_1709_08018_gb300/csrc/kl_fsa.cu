@@ -65,25 +65,6 @@ struct FsaShared {
   unsigned long long ways[kFsaMaxDepth + 1][kFsaStates];
 };
 
-// One map in FP64 (a refined reciprocal instead of divisions), its multiply-adds
-// spelled out so that every string's value has the same bits wherever the
-// compiler inlines it.
-__device__ __forceinline__ double mul_sub(double a, double b, double c, double d) {
-  return __fma_rn(a, b, -__dmul_rn(c, d));
-}
-__device__ __forceinline__ double mul_add(double a, double b, double c, double d) {
-  return __fma_rn(a, b, __dmul_rn(c, d));
-}
-__device__ __forceinline__ dc fsa_map(const double* M, dc z) {
-  const dc num = {__dadd_rn(mul_sub(M[0], z.re, M[1], z.im), M[2]),
-                  __dadd_rn(mul_add(M[0], z.im, M[1], z.re), M[3])};
-  const dc den = {__dadd_rn(mul_sub(M[4], z.re, M[5], z.im), M[6]),
-                  __dadd_rn(mul_add(M[4], z.im, M[5], z.re), M[7])};
-  const double r = rcp64(mul_add(den.re, den.re, den.im, den.im));
-  return {__dmul_rn(mul_add(num.re, den.re, num.im, den.im), r),
-          __dmul_rn(mul_sub(num.im, den.re, num.re, den.im), r)};
-}
-
 // Pixel of map M of the point z (as FP32: zr, zi) where an FP32 evaluation
 // settles it, -1 for certainly outside the window, kUnsettled otherwise.
 // Error: numerator and denominator are sums of products of once-rounded
@@ -154,7 +135,7 @@ __device__ __forceinline__ void fsa_word(FsaWalk& w, dc z) {
 __device__ __forceinline__ void fsa_drain(FsaWalk& w, uint32_t n) {
   __syncwarp();
   const uint32_t lane = threadIdx.x & 31, k = w.len - n + lane;
-  if (lane < n) fsa_word(w, fsa_map(w.S->g + 8 * w.Q->x[k], {w.Q->zr[k], w.Q->zi[k]}));
+  if (lane < n) fsa_word(w, point_map(w.S->g + 8 * w.Q->x[k], {w.Q->zr[k], w.Q->zi[k]}));
   w.len -= n;
   __syncwarp();
 }
@@ -198,7 +179,7 @@ __device__ __forceinline__ void fsa_walk(FsaWalk& w, bool on, uint32_t state, dc
     for (uint32_t k = 0; k < w.most; ++k) {
       const bool child = k < n;
       const uint32_t x = child ? S.sym[state][k] : 0u;
-      fsa_walk<h - 1>(w, child, child ? S.to[state][k] : 0u, fsa_map(S.g + 8 * x, z));
+      fsa_walk<h - 1>(w, child, child ? S.to[state][k] : 0u, point_map(S.g + 8 * x, z));
     }
   }
 }
@@ -258,7 +239,7 @@ __global__ void __launch_bounds__(kFsaThreads) fsa_render_kernel(
       const uint32_t x = S.sym[state][i];
       state = S.to[state][i];
       if (k == 0) z = {S.seed[2 * x], S.seed[2 * x + 1]};
-      z = fsa_map(S.g + 8 * x, z);
+      z = point_map(S.g + 8 * x, z);
     }
     fsa_walk<h>(w, on, state, z);
   }

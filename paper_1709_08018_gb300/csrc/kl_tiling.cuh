@@ -31,12 +31,10 @@ namespace {
 constexpr uint32_t kShortTiling = 9;
 constexpr int kShortWalk = 2;
 
+// Its multiply-adds are spelled out so that a word has the same value, bit for bit,
+// wherever it is evaluated (from its seed, or as a walk's first or second letter).
 __device__ __forceinline__ dc short_map(const Group& G, int x, dc z) {
-  const double* M = G.g + 8 * x;
-  const dc num = {M[0] * z.re - M[1] * z.im + M[2], M[0] * z.im + M[1] * z.re + M[3]};
-  const dc den = {M[4] * z.re - M[5] * z.im + M[6], M[4] * z.im + M[5] * z.re + M[7]};
-  const double rc = rcp64(den.re * den.re + den.im * den.im);
-  return {(num.re * den.re + num.im * den.im) * rc, (num.im * den.re - num.re * den.im) * rc};
+  return point_map(G.g + 8 * x, z);
 }
 
 // Roots of the walk: the words of lengths 1 .. short_root_length; those of the
