@@ -12,8 +12,8 @@ at length 18 (4096^2) as secondary keys, each with its own IoU and error.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
-Rank 0 prints one JSON line.  With N > 1 (torchrun, one process per GPU) the
-job is sharded: rank k renders shard k of N (kl_params.shard_index /
+Rank 0 prints one JSON line (the whole record goes to stderr: print_line).
+With N > 1 (torchrun, one process per GPU) the job is sharded: rank k renders shard k of N (kl_params.shard_index /
 shard_count, a partition of the words by prefix slot) into its own image, and
 one reduce sums the uint32 images and the counters onto rank 0 inside the
 timed region (strong scaling: value = the job's words / the slowest rank's
@@ -1120,10 +1120,37 @@ def run_ours(args):
             line["lod"]["speedup_over_fp64_render"] = (
                 line["lod"]["words_per_s_pruned"] / fp64_2["words_per_s"])
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        print_line(line)
     if world > 1:
         import torch.distributed as dist
         dist.destroy_process_group()
+
+
+# The headline and what it is checked with: on the line as they are.
+EXACT_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "config",
+              "clocks", "roofline", "e2e", "cpu_baseline", "accuracy", "counters")
+# Legs and tables of the stderr record alone.
+SIDE_LEGS = ("fp64_gasket_d10", "paper_scan", "maskit_example", "multiseed")
+TABLES = ("valid_settings", "per_group")
+
+
+def short(x):
+    """x with floats rounded to 6 significant digits, without its descriptions
+    (texts of more than 50 letters) and tables."""
+    if isinstance(x, float):
+        return float(f"{x:.6g}")
+    if isinstance(x, dict):
+        return {k: short(v) for k, v in x.items()
+                if k not in TABLES and not (isinstance(v, str) and len(v) > 50)}
+    return [short(v) for v in x] if isinstance(x, (list, tuple)) else x
+
+
+def print_line(line):
+    """The result as one line on stdout, short enough for a reader that keeps 8,000
+    letters; the whole record, descriptions and tables too, as one on stderr."""
+    print(json.dumps(line), file=sys.stderr, flush=True)
+    print(json.dumps({k: v if k in EXACT_KEYS else short(v) for k, v in line.items()
+                      if k not in SIDE_LEGS}), flush=True)
 
 
 def main():
