@@ -13,11 +13,12 @@ at length 18 (4096^2) as secondary keys, each with its own IoU and error.
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
 Rank 0 prints one JSON line (the whole record goes to stderr: print_line).
-With N > 1 (torchrun, one process per GPU) the job is sharded: rank k renders shard k of N (kl_params.shard_index /
-shard_count, a partition of the words by prefix slot) into its own image, and
-one reduce sums the uint32 images and the counters onto rank 0 inside the
-timed region (strong scaling: value = the job's words / the slowest rank's
-time).  The oracle legs (CPU baseline and accuracy) run at N = 1 only.
+With N > 1 (torchrun, one process per GPU) the job is sharded: rank k renders
+shard k of N (kl_params.shard_index / shard_count, a partition of the words by
+prefix slot) into its own image, and one reduce sums the uint32 images and the
+counters onto rank 0 inside the timed region (strong scaling: value = the
+job's words / the slowest rank's time).  The oracle legs (CPU baseline and
+accuracy) run at N = 1 only.
 """
 import argparse
 import hashlib
@@ -359,10 +360,10 @@ def tiling_config(kl, dev, steps: int, flush):
 
 
 def scan_config(kl, dev, flush):
-    """The paper's own enumeration for a general presentation (kl_render_fsa):
-    the unpruned 4-ary tree of depth 14 of the gasket group scanned and
-    filtered by the indexed Cayley table, FP64, against the reduced-index
-    render of the same words (FP64 and mixed)."""
+    """The paper's words of a general presentation (kl_render_fsa): the strings
+    of 14 letters that the indexed Cayley table of the gasket group keeps out of
+    the unpruned 4-ary tree, FP64, against the reduced-index render of the
+    same words (FP64 and mixed)."""
     import torch
     d, W = 14, 4096
     window = (-1.5, 1.5, -1.5, 1.5)
@@ -395,22 +396,20 @@ def scan_config(kl, dev, flush):
     rm = kl.Renderer(pm, device=dev)
     reduced_mixed_ms = timed(lambda: rm())
     return {"workload": "gasket ta=tb=2, the strings of 14 letters that the indexed Cayley "
-                        "table keeps out of 4^14 (walked as a tree; strings_per_s counts "
-                        "all 4^14), FP64, 4096^2",
-            "strings": 4 ** d, "kept_words": kept, "ms": scan_ms,
-            "strings_per_s": 4 ** d / (scan_ms / 1000.0),
+                        "table keeps (walked as a tree, no other string is looked at), "
+                        "FP64, 4096^2",
+            "kept_words": kept, "ms": scan_ms,
             "kept_words_per_s": kept / (scan_ms / 1000.0),
             "reduced_index_fp64_ms": reduced64_ms, "reduced_index_mixed_ms": reduced_mixed_ms,
-            "speedup_reduced_index_mixed_over_scan": scan_ms / reduced_mixed_ms}
+            "speedup_reduced_index_mixed_over_table": scan_ms / reduced_mixed_ms}
 
 
 def maskit_config(kl, dev, flush):
     """The paper's example: Maskit's slice at mu = -0.097 + 1.838i, depth 14,
-    tiling mode (every node of the tree, all lengths 1..14).  The paper's way:
-    scan all 4^k strings of every length k (357,913,940 in all) and filter by
-    the indexed Cayley table (kl_render_fsa, FP64); the indexed way: decode
-    only the 2 (3^14 - 1) reduced words (kl_render, tiling mode, FP64 and
-    mixed).  One period of the limit set, 4096^2."""
+    tiling mode (every node of the tree, all lengths 1..14).  By the indexed
+    Cayley table: the strings of every length k that it keeps out of 4^k
+    (kl_render_fsa, FP64, one call per length); by index: the 2 (3^14 - 1)
+    reduced words (kl_render, tiling mode, FP64, double-float and mixed).  One period of the limit set, 4096^2."""
     import torch
     d, W = 14, 4096
     window = (-1.0, 1.0, -0.08, 1.92)
@@ -437,17 +436,16 @@ def maskit_config(kl, dev, flush):
           for k in range(1, d + 1)]
     f = kl.fsa_from_params(table, pk[0])
 
-    def scan_all_lengths():
+    def all_lengths():
         for p in pk:
             kl.render_fsa(f, p, img, cnt)
-    scan_ms = timed(scan_all_lengths)
+    scan_ms = timed(all_lengths)
     scan_img = img.clone()
     nodes = 2 * (3 ** d - 1)
     assert int(cnt[0].item()) + int(cnt[1].item()) == nodes
     out = {"workload": "Maskit mu = -0.097+1.838i, depth 14, tiling mode (all lengths 1..14), "
                        "window [-1,1]x[-0.08,1.92], 4096^2",
-           "nodes": nodes, "strings_scanned": sum(4 ** k for k in range(1, d + 1)),
-           "paper_scan_fp64_ms": scan_ms}
+           "nodes": nodes, "by_table_fp64_ms": scan_ms}
     for name, prec in (("fp64", kl.FP64), ("df64", kl.DF64), ("mixed", kl.MIXED)):
         p = kl.params_group(gens, seeds8, d, W, W, window, prec, mode=kl.TILING)
         r = kl.Renderer(p, device=dev)
@@ -455,9 +453,9 @@ def maskit_config(kl, dev, flush):
         if name in ("fp64", "df64"):
             diff = int((r.image.to(torch.int64) - scan_img.to(torch.int64)).abs().sum().item())
             out[f"{name}_images_differ_in_hits"] = diff
-    out["speedup_indexed_fp64_over_scan"] = scan_ms / out["indexed_fp64_ms"]
-    out["speedup_indexed_df64_over_scan"] = scan_ms / out["indexed_df64_ms"]
-    out["speedup_indexed_mixed_over_scan"] = scan_ms / out["indexed_mixed_ms"]
+    out["speedup_indexed_fp64_over_table"] = scan_ms / out["indexed_fp64_ms"]
+    out["speedup_indexed_df64_over_table"] = scan_ms / out["indexed_df64_ms"]
+    out["speedup_indexed_mixed_over_table"] = scan_ms / out["indexed_mixed_ms"]
     return out
 
 
@@ -1136,12 +1134,12 @@ TABLES = ("valid_settings", "per_group")
 
 def short(x):
     """x with floats rounded to 6 significant digits, without its descriptions
-    (texts of more than 50 letters) and tables."""
+    (texts of more than 45 letters) and tables."""
     if isinstance(x, float):
         return float(f"{x:.6g}")
     if isinstance(x, dict):
         return {k: short(v) for k, v in x.items()
-                if k not in TABLES and not (isinstance(v, str) and len(v) > 50)}
+                if k not in TABLES and not (isinstance(v, str) and len(v) > 45)}
     return [short(v) for v in x] if isinstance(x, (list, tuple)) else x
 
 
