@@ -60,7 +60,8 @@ typedef enum {
 
 /* Arithmetic of the per-word work. */
 typedef enum {
-  KL_FP64 = 0,   /* every step in FP64 */
+  KL_FP64 = 0,   /* every step in FP64 (renders: every word in the pixel of its FP64
+                    value, most settled in FP32 with an error bound) */
   KL_MIXED = 1,  /* prefix products, renormalisation and near-parabolic words in
                     FP64; the per-word map in FP32 in a per-prefix local frame */
   KL_DF64 = 2    /* prefix products, tables and pole-form constants in FP64; the
@@ -68,11 +69,11 @@ typedef enum {
                     value an unevaluated sum of two floats, about 48 significant bits,
                     error-free sums and products built from FP32 adds and fused
                     multiply-adds), giving word values within the FP64 tolerance
-                    (1e-9 relative) at FP32-pipe speed, 117 FP32 operations per word.  Prefixes whose pole form is
-                    invalid or out of float range (P10 ~ 0, pixel offsets >= 2^20,
-                    constants outside [1e-30, 1e30]) run in FP64.  kl_render (limit
-                    set and tiling), kl_render_noalloc and kl_eval_words only; not
-                    with cull = 1 */
+                    (1e-9 relative) at FP32-pipe speed, 117 FP32 operations per word.
+                    Prefixes whose pole form is invalid or out of float range
+                    (P10 ~ 0, pixel offsets >= 2^20, constants outside
+                    [1e-30, 1e30]) run in FP64.  kl_render (limit set and tiling),
+                    kl_render_noalloc and kl_eval_words only; not with cull = 1 */
 } kl_precision;
 
 /* Which words a render draws (Sec. "Implementation": the two drawing modes). */
@@ -163,7 +164,9 @@ typedef struct {
 enum {
   KL_CNT_IN_WINDOW = 0,    /* words drawn into the image */
   KL_CNT_DROPPED = 1,      /* words outside the window or non-finite */
-  KL_CNT_FP64_WORDS = 2,   /* KL_MIXED, KL_DF64: words evaluated on the FP64 path */
+  KL_CNT_FP64_WORDS = 2,   /* KL_MIXED, KL_DF64: words whose prefix is on the FP64 path
+                              (their pixel is the FP64 map's; most are settled in FP32
+                              with an error bound) */
   KL_CNT_ATOMICS = 3,      /* image atomics issued (after run-length merging) */
   KL_N_COUNTERS = 4
 };
@@ -475,7 +478,8 @@ KL_API int kl_fsa_count(const kl_fsa* f, uint32_t depth, uint64_t* count);
 /* Render of the kept strings of depth p->depth with the view, image size and
  * accumulate flag of *p (its gens, seeds and mode are not used; precision
  * must be KL_FP64).  Counters as kl_render (KL_CNT_FP64_WORDS = kept words).
- * d_workspace: at least KL_FSA_WORKSPACE_BYTES, 256-byte aligned. */
+ * d_workspace: at least KL_FSA_WORKSPACE_BYTES, 256-byte aligned; checked, but
+ * nothing reads or writes it (kept for callers of the scan that did). */
 KL_API int kl_render_fsa(const kl_fsa* f, const kl_params* p, uint32_t* d_image,
                          uint64_t* d_counters, void* d_workspace, size_t workspace_bytes,
                          void* stream);
@@ -512,8 +516,7 @@ KL_API int kl_render_noalloc(const kl_params* p, uint32_t* d_image, uint64_t* d_
 
 /* Instrumentation: when set, kl_render records the CUDA events ev_start and
  * ev_stop (cudaEvent_t, created by the caller) on its stream immediately
- * before and after its main per-word kernel (the FP64 or mixed render
- * kernel), so that the caller can time that kernel alone with
+ * before and after its main per-word kernel, so that the caller can time that kernel alone with
  * cudaEventElapsedTime.  NULL, NULL switches it off.  The setting belongs to
  * the calling host thread and applies to every following kl_render call made
  * from that thread (other threads are not affected).  This is an

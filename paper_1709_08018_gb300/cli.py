@@ -122,8 +122,8 @@ def run_batch(a, kl, klsynth, torch):
 
 
 def run_scan(a, kl, klsynth, torch):
-    """The paper's scan (kl_render_fsa) of the gasket group with the torus
-    table: all 4^d strings of depth d (default 14), FP64, 4096^2."""
+    """The strings of the paper's scan (kl_render_fsa) of the gasket group that the
+    torus table keeps out of the 4^d of depth d (default 14), FP64, 4096^2."""
     d = a.depth or 14
     W = a.size or 4096
     table = [[0, 1, 2, 3, 4], [1, 1, 2, 0, 4], [2, 1, 2, 3, 0], [3, 0, 2, 3, 4], [4, 1, 0, 3, 4]]
@@ -139,7 +139,7 @@ def run_scan(a, kl, klsynth, torch):
         e1.record()
     torch.cuda.synchronize()
     c = cnt.cpu().tolist()
-    print(f"scan d={d}: strings {4 ** d}, kept {c[2]}, in-window {c[0]}, "
+    print(f"scan d={d}: kept {c[2]} of {4 ** d} strings, in-window {c[0]}, "
           f"{e0.elapsed_time(e1):.3f} ms")
 
 

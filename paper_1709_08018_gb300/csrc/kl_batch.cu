@@ -100,7 +100,8 @@ __global__ void __launch_bounds__(BT, 1280 / BT) batch_mixed_kernel(
         const uint32_t g = (uint32_t)(ent >> 32), slot = (uint32_t)(ent & 0xFFFFFFFFull);
         const Tables T = D[g].T;
         const UnitTally r = fallback_unit(T.pre64, T.flags, T.suf64, T.pre32, T.suf32p, slot,
-                                          rem / cmax, rem % cmax, D[g].L.np, D[g].L.ns, D[g].V, D[g].img);
+                                          rem / cmax, rem % cmax, D[g].L.np, D[g].L.ns, D[g].V,
+                                          D[g].img);
         if (r.words) {
           unsigned long long* c = D[g].cnt;
           atomicAdd(c + KL_CNT_IN_WINDOW, (unsigned long long)r.in_window);

@@ -44,7 +44,7 @@ constexpr uint32_t kNearPar = 2u;    // |tr^2 - 4 det| small: near-parabolic (cu
 constexpr uint32_t kWide = 4u;       // local FP32 frame unsafe (far or huge offsets)
 constexpr uint32_t kFallback = 8u;   // KL_MIXED, KL_DF64: words of this prefix run in FP64
 constexpr uint32_t kDfRange = 16u;   // a pole-form constant outside the double-float range
-constexpr uint32_t kNoFilter = 32u;  // no filter constants: words take the exact map (kl_filter.cuh)
+constexpr uint32_t kNoFilter = 32u;  // no filter constants: exact map (kl_filter.cuh)
 constexpr uint32_t kOnFp32 = 64u;    // KL_MIXED: words on the FP32 map (its record is pre32's)
 constexpr uint32_t kNear32 = 128u;   // words on the FP64 map, with an FP32 record for certified
                                      // tests (culled and mixed renders)
@@ -764,7 +764,8 @@ __device__ void combine_entry(const View& V, const Plan& L, double ptol, int pre
     else
       R.fl |= kNoFilter;
   } else {
-    if ((what >= kCullTables || prec == KL_MIXED) && !(R.fl & (kOnFp32 | kDirect | kWide))) R.fl |= kNear32;
+    if ((what >= kCullTables || prec == KL_MIXED) && !(R.fl & (kOnFp32 | kDirect | kWide)))
+      R.fl |= kNear32;
     if (R.fl & (kOnFp32 | kNear32)) T.pre32[slot] = pre32_of(R.c64);
   }
   T.flags[slot] = R.fl;
@@ -1011,8 +1012,8 @@ __device__ __forceinline__ void near_words64(const Pre32& k, const Pre64* __rest
     const int vl = __float_as_int(__fadd_rd(v - E, magic));
     const int vh = __float_as_int(__fadd_rd(v + E, magic));
     int pix;
-    if (m > 1e-30f && m < 1e30f && q < 0.25f && E < 0.25f && fabsf(u) < 0x1p20f && fabsf(v) < 0x1p20f && ul == uh &&
-        vl == vh) {
+    if (m > 1e-30f && m < 1e30f && q < 0.25f && E < 0.25f && fabsf(u) < 0x1p20f &&
+        fabsf(v) < 0x1p20f && ul == uh && vl == vh) {
       const int col = ul - k.kx, row = vl - k.ky;
       pix = ((uint32_t)col < V.W && (uint32_t)row < V.H) ? row * (int)V.W + col : -1;
     } else {
@@ -1025,10 +1026,11 @@ __device__ __forceinline__ void near_words64(const Pre32& k, const Pre64* __rest
   }
 }
 
-// Mixed-mode FP64 fallback unit (kept out of line so that its registers do
-// not bind the FP32 loop; FP32 with a bound first: gasket, 14 letters, 1024 x 519,
-// 78 -> 44 us, the fallback words had kept the FP64 pipe busy after the others): (fallback prefix, one of its three suffix letters,
-// a chunk of fb_chunk suffix points).  Chunks past the end are empty.
+// Mixed-mode FP64 fallback unit: a fallback prefix, one of its three suffix
+// letters, a chunk of fb_chunk suffix points.  Chunks past the end are empty.  Kept
+// out of line so that its registers do not bind the FP32 loop.  Its words are tried
+// in FP32 first (gasket, 14 letters, 1024 x 519: 78 -> 44 us; all in FP64 they kept
+// that pipe busy after the others had ended).
 template <bool BBOX = false>
 __device__ __noinline__ UnitTally fallback_unit(const Pre64* __restrict__ pre,
                                                 const uint32_t* __restrict__ flags,

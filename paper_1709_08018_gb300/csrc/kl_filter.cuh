@@ -17,8 +17,8 @@ namespace {
 // map alone gives.  The FP64 pipe has 2 lanes per SM against 128 of the FP32
 // pipe, and the double-float map takes 117 FP32 operations; taking them out of
 // the loop is what this buys.  Near-cusp group, length 20, 8192^2: FP64
-// 104.9 -> 3.4 ms, double-float 18.3 -> 3.5 ms; gasket, length 18, 4096^2:
-// 11.74 -> 0.42 and 2.06 -> 0.44 ms (whole renders, the same images).
+// 104.9 -> 3.3 ms, double-float 18.3 -> 3.4 ms; gasket, length 18, 4096^2:
+// 11.74 -> 0.40 and 2.06 -> 0.44 ms (whole renders, the same images).
 //
 // Map.  With z = alpha + beta/(v + gamma), one complex scale k = 1/(sx beta)
 // gives omega = k v + g, g = k gamma, and the offset from alpha in x-pixel
@@ -31,8 +31,9 @@ namespace {
 // outside one window side, in either case cut to |offset| <= 8 rho, rho the
 // offset of the word that opened it.  Words inside the box extend its run; an
 // outside box is large, so the words outside the window (a third of the
-// near-cusp group's) hardly ever end a run: 5% of the warp's pair steps meet
-// a run end there against 25% with one-pixel runs.
+// near-cusp group's) hardly ever end a run.  Runs that end inside cost an image
+// add each: 1.09e7 adds in 7.3e7 warp steps at length 20, 8192^2, 2.8e6 in 2.7e6 at
+// length 17, 4096^2, where a run end of some lane falls in nearly every step.
 //
 // Error bound, eps = 2^-24.  |delta omega| <= eps (11 |omega| + 8 |g|): k is
 // the FP32 reciprocal of the FP32-rounded constant (6 eps, common to k v and

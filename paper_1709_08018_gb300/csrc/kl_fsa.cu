@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(kFsaThreads) fsa_render_kernel(
 
 using FsaKernel = void (*)(FsaDev, View, uint32_t*, unsigned long long*);
 
-int fsa_check(const kl_fsa* f, uint32_t d, unsigned long long* n_idx) {
+int fsa_check(const kl_fsa* f, uint32_t d) {
   if (!f || f->m < 1 || f->m > KL_FSA_MAX_LETTERS) return KL_EINVAL;
   if (d < 1 || d > (uint32_t)kFsaMaxDepth) return KL_ERANGE;
   const uint32_t m = f->m;
@@ -265,7 +265,6 @@ int fsa_check(const kl_fsa* f, uint32_t d, unsigned long long* n_idx) {
     if (n > (1ull << 40) / m) return KL_ERANGE;
     n *= m;
   }
-  *n_idx = n;
   return KL_OK;
 }
 
@@ -289,8 +288,7 @@ void fsa_ways(const kl_fsa* f, uint32_t depth,
 }  // namespace
 
 extern "C" int kl_fsa_count(const kl_fsa* f, uint32_t depth, uint64_t* count) {
-  unsigned long long n_idx = 0;
-  const int st = fsa_check(f, depth, &n_idx);
+  const int st = fsa_check(f, depth);
   if (st != KL_OK) return st;
   if (!count) return KL_EINVAL;
   unsigned long long ways[kFsaMaxDepth + 1][kFsaStates];
@@ -304,8 +302,7 @@ extern "C" int kl_render_fsa(const kl_fsa* f, const kl_params* p, uint32_t* d_im
                              void* stream) {
   if (!p || !d_image || !valid_view(p)) return KL_EINVAL;
   if (p->precision != KL_FP64) return KL_EINVAL;
-  unsigned long long n_idx = 0;
-  int st = fsa_check(f, p->depth, &n_idx);
+  const int st = fsa_check(f, p->depth);
   if (st != KL_OK) return st;
   if (!d_workspace || ((uintptr_t)d_workspace & 255u) != 0) return KL_EINVAL;
   if (workspace_bytes < KL_FSA_WORKSPACE_BYTES) return KL_ENOSPACE;

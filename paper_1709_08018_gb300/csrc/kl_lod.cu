@@ -136,7 +136,7 @@ __device__ __forceinline__ bool resolved(int4 b, int W, int H, int ext) {
 // labels
 
 // The exact mixed (or FP64) render with per-slot pixel boxes; one persistent
-// launch like render_mixed_kernel / render64_kernel.
+// launch like render_mixed_kernel; FP64 words all by the FP64 map.
 template <int BT, bool MIXED>
 __global__ void __launch_bounds__(BT, 1536 / BT) lod_exact_kernel(
     Tables T, Plan L, View V, Work Wk, BoxRef B, uint32_t* __restrict__ img,
@@ -156,7 +156,8 @@ __global__ void __launch_bounds__(BT, 1536 / BT) lod_exact_kernel(
         const uint32_t e = unit / (3u * chunks), rem = unit % (3u * chunks);
         const uint32_t slot = (uint32_t)(T.fb[e] & 0xFFFFFFFFull);
         const UnitTally r = fallback_unit<true>(T.pre64, T.flags, T.suf64, T.pre32, T.suf32p,
-                                                slot, rem / chunks, rem % chunks, L.np, L.ns, V, img, B);
+                                                slot, rem / chunks, rem % chunks, L.np, L.ns, V,
+                                                img, B);
         words += r.words;
         fp64_words += r.words;
         t.in_window += r.in_window;

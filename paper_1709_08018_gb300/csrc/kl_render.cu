@@ -1,6 +1,7 @@
 // Single render, decode and evaluation entry points of the C ABI (sm_103a).
 // The arithmetic, tables and per-item bodies are in kl_common.cuh and the
-// headers it includes (kl_df.cuh, kl_cull.cuh, kl_plan.cuh).
+// headers it includes (kl_df.cuh, kl_filter.cuh, kl_cull.cuh, kl_plan.cuh); the
+// tiling render's are in kl_tiling.cuh.
 #include <cmath>
 #include <mutex>
 
@@ -368,7 +369,8 @@ int launch_render(const kl_params* p, const Plan& L, const View& V, const Tables
     if (launch_dependent(disk_kernel, dim3((warps + 3u) / 4u), dim3(128), s, L, T, sized) != KL_OK)
       return KL_ECUDA;
     const bool mixed = p->precision == KL_MIXED;
-    const void* k = mixed ? (const void*)cull_kernel<BT, true> : (const void*)cull_kernel<BT, false>;
+    const void* k =
+        mixed ? (const void*)cull_kernel<BT, true> : (const void*)cull_kernel<BT, false>;
     if (device_slots(k, BT, &sms, &occ) != KL_OK) return KL_ECUDA;
     // warp-sized items: 32 prefixes x a chunk of top-level blocks (one by default)
     const Work Wk = make_work(L, 32, L.cnb[L.clev - 1], sms * occ * (BT / 32),
