@@ -794,7 +794,7 @@ def fp_peaks():
             SMS * FP64_LANES_PER_SM * sm_max * 1e6 / 1e12)
 
 
-def roofline_filter(words, kern_ms, wl, exact_ops):
+def roofline_filter(words, kern_ms, wl, exact_ops, traffic_key):
     """FP64 and double-float renders: every word takes the FP32 filter, about
     one in 10^4 the exact map of `exact_ops` operations (not counted)."""
     fp32_peak = fp_peaks()[0]
@@ -803,11 +803,11 @@ def roofline_filter(words, kern_ms, wl, exact_ops):
             "unit": "T FP32-op/s", "frac": ach / fp32_peak,
             "peak_kind": "derived: 152 SMs x 128 FP32 lanes x max SM clock",
             "filter_ops_per_word": FILTER_OPS_PER_WORD, "ops_per_word": exact_ops,
-            "traffic": traffic_for("render_words_kernel", wl), "kernel_ms": kern_ms}
+            "traffic": traffic_for(traffic_key, wl), "kernel_ms": kern_ms}
 
 
 def roofline64(words, kern_ms, wl):
-    return roofline_filter(words, kern_ms, wl, FP64_OPS_PER_WORD)
+    return roofline_filter(words, kern_ms, wl, FP64_OPS_PER_WORD, "render_words_kernel<fp64>")
 
 
 def plain_fp64(kl, cfg, dev, flush, K=3):
@@ -840,7 +840,7 @@ def roofline32(words_fp32, kern_ms, wl):
 
 
 def roofline_df(words_df, kern_ms, wl):
-    return roofline_filter(words_df, kern_ms, wl, DF64_OPS_PER_WORD)
+    return roofline_filter(words_df, kern_ms, wl, DF64_OPS_PER_WORD, "render_words_kernel<df64>")
 
 
 def secondary(kl, cfg, prec, flush, stream, dev, K):
