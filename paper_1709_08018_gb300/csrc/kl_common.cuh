@@ -676,6 +676,11 @@ __device__ __forceinline__ void prefix_rec(const View& V, const Plan& L, double 
 // them costs 7 us (length 14, 324 slots, 1000 x 507: 81 against 74 us); from 8,748
 // on (length 18) it pays.
 constexpr uint32_t kMinSizeSlots = 8192;
+// Nor does it pay past kMaxSizeSlots (length 21 and more: 708,588 slots of length 24
+// are as many adds on some twenty addresses, 14.7 against 13.5 ms; length 22, 1024^2,
+// up to 14% slower) or with suffixes of fewer than kMinSizePoints points (length 16,
+// 9 prefix letters: 10 to 34% slower but for the near-cusp group).
+constexpr uint32_t kMaxSizeSlots = 65536, kMinSizePoints = 6561;
 __device__ __forceinline__ uint32_t size_class(const Pre64& c, uint32_t flags) {
   if (flags & kDirect) return 0u;
   const int e = (int)(max(abs_hi(c.c1), abs_hi(c.c2)) >> 20) - 1023;

@@ -354,7 +354,9 @@ WordsKernel words_kernel(uint32_t precision) {
 
 // What the combine pass of a culled render of plan L prepares.
 WordTables cull_tables(const Plan& L) {
-  return 4u * L.np >= kMinSizeSlots ? kSizeTables : kCullTables;
+  const bool sized =
+      4u * L.np >= kMinSizeSlots && 4u * L.np < kMaxSizeSlots && L.ns >= kMinSizePoints;
+  return sized ? kSizeTables : kCullTables;
 }
 
 template <int BT>
