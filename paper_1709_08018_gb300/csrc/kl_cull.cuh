@@ -480,6 +480,11 @@ struct CullWarp {
 // 2055: 277 -> 189 us (mixed), 716 -> 183 us in FP64 together with the FP32 tests
 // above, which also take the near-cusp group at length 20, 8192 x 4103, from 3.76
 // to 0.64 ms in FP64 (mixed: 0.51 before and after, few of its words are FP64).
+// From kSlotOrderBlocks prefix blocks per letter on (length 21) items go letter by
+// letter in slot order: neighbours share their tables and their part of the image,
+// and the end of so long a queue is short (mixed, 4096^2: length 22 1559 -> 1500 us,
+// length 24 14.18 -> 13.53 ms).
+constexpr uint32_t kSlotOrderBlocks = 512;
 __device__ __forceinline__ uint32_t cull_block_order(uint32_t i, uint32_t n) {
   if (i == 0 || n < 4) return i;
   const uint32_t mid = (n - 1) / 2;
@@ -496,11 +501,18 @@ __device__ __forceinline__ void cull_item(CullWarp<MIXED>& w, uint32_t item, con
                                           const Plan& L, const View& V, const Tables& T,
                                           uint32_t* __restrict__ img, uint32_t top_blocks,
                                           bool sized = false) {
-  // prefix blocks slowest, suffix blocks fastest
-  const uint32_t c = item % Wk.n_chunks, t = item / Wk.n_chunks;
-  const uint32_t q = t % 12u, pb = sized ? t / 12u : cull_block_order(t / 12u, Wk.n_pb);
-  const int x = (int)(q / 3u);
-  const int u = allowed_letter((int)(q % 3u), (x + 2) & 3);
+  int x, u;
+  uint32_t pb, c;
+  if (Wk.n_pb >= kSlotOrderBlocks) {
+    item_of(item, Wk, x, u, pb, c);
+  } else {
+    // prefix blocks slowest, suffix blocks fastest
+    c = item % Wk.n_chunks;
+    const uint32_t t = item / Wk.n_chunks, q = t % 12u;
+    pb = sized ? t / 12u : cull_block_order(t / 12u, Wk.n_pb);
+    x = (int)(q / 3u);
+    u = allowed_letter((int)(q % 3u), (x + 2) & 3);
+  }
   const uint32_t k = pb * 32 + w.lane;
   uint32_t slot = (uint32_t)x * L.np + L.r0 + k;
   const bool live = k < L.nr;
