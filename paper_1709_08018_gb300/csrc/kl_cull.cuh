@@ -57,7 +57,10 @@ constexpr int kUncertified = -2;
 // EXACT64: the block of a prefix whose words run in FP64 (k: its constants
 // rounded to FP32, D already widened by near_slack).  The rounding of the other
 // constants and of this test's own steps is below 16 eps of |M| / |w|, both
-// axes alike, eps = 2^-24; the code takes 32.
+// axes alike, eps = 2^-24; the code takes 32.  Beside these and the offsets' share
+// only the rounding of alpha's fraction is left, 2^-25 px; 2^-21 are taken (with the
+// 2^-11 of the mixed map a limit set of a few pixels was hardly certified: FP64, 14
+// letters, the set a hundredth of a pixel across its edge, 57 -> 41 us).
 template <bool EXACT64 = false>
 __device__ __forceinline__ int block_pixel32(const Pre32& k, float nrm, float4 D, const View& V) {
   const float c0r = D.x + k.gr, c0i = D.y + k.gi;
@@ -67,7 +70,7 @@ __device__ __forceinline__ int block_pixel32(const Pre32& k, float nrm, float4 D
   const float X = fmaf(fmaf(k.c1, c0r, k.c2 * c0i), rq, k.axf);
   const float Y = fmaf(fmaf(k.c3, c0r, k.c4 * c0i), rq, k.ayf);
   const float R = nrm * D.z * rq;
-  float m = R + fmaf(fabsf(X) + fabsf(Y) + R, 0x1p-20f, 0x1p-11f);
+  float m = R + fmaf(fabsf(X) + fabsf(Y) + R, 0x1p-20f, EXACT64 ? 0x1p-21f : 0x1p-11f);
   if (EXACT64) {
     if (!(n2 > 1e-30f && n2 < 1e30f)) return kUncertified;
     m = fmaf(nrm * sqrtf(n2) * rq, 0x1p-19f, m);
