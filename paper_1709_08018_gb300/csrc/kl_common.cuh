@@ -48,6 +48,8 @@ constexpr uint32_t kNoFilter = 32u;  // no filter constants: exact map (kl_filte
 constexpr uint32_t kOnFp32 = 64u;    // KL_MIXED: words on the FP32 map (its record is pre32's)
 constexpr uint32_t kNear32 = 128u;   // words on the FP64 map, with an FP32 record for certified
                                      // tests (culled and mixed renders)
+constexpr uint32_t kFar32 = 256u;    // kNear32, but too far from the window for a word in it to
+                                     // be settled in FP32: words take the FP64 map
 
 // What the words of a render read beside the FP64 records (combine_entry).
 enum WordTables : int {
@@ -771,7 +773,15 @@ __device__ void combine_entry(const View& V, const Plan& L, double ptol, int pre
   } else {
     if ((what >= kCullTables || prec == KL_MIXED) && !(R.fl & (kOnFp32 | kDirect | kWide)))
       R.fl |= kNear32;
-    if (R.fl & (kOnFp32 | kNear32)) T.pre32[slot] = pre32_of(R.c64);
+    if (R.fl & (kOnFp32 | kNear32)) {
+      const Pre32 k = pre32_of(R.c64);
+      T.pre32[slot] = k;
+      // a word in the window then has an offset R >= 2^16 px, and 64 eps R >= 1/4
+      // settles nothing (near_words64); mixed, 15 letters, a view of 4e-5: 369 -> 324 us
+      if ((R.fl & kNear32) && (k.axi < -65536 || k.axi > (int)V.W + 65536 ||
+                               k.ayi < -65536 || k.ayi > (int)V.H + 65536))
+        R.fl |= kFar32;
+    }
   }
   T.flags[slot] = R.fl;
   if (what == kSizeTables) atomicAdd(size_counts(L, T) + 32 * x + size_class(R.c64, R.fl), 1u);
@@ -1052,7 +1062,7 @@ __device__ __noinline__ UnitTally fallback_unit(const Pre64* __restrict__ pre,
   const uint32_t j1 = min(ns, j0 + len);
   Tally t;
   const uint32_t fl = flags[slot];
-  if (!BBOX && (fl & kNear32)) {
+  if (!BBOX && (fl & (kNear32 | kFar32)) == kNear32) {
     const Pre32 k32 = pre32[slot];
     // the Frobenius norm bounds the operator norm
     const float nrm = sqrtf(fmaf(k32.c1, k32.c1, k32.c2 * k32.c2) +

@@ -360,7 +360,7 @@ struct CullWarp {
     const uint32_t j0 = b * C->sz[l];
     if (MIXED && !f64) {
       mixed_block_words(slot, (int)u, j0, C->sz[l], L, V, T, t, words, img);
-    } else if (T.flags[slot] & kNear32) {
+    } else if ((T.flags[slot] & (kNear32 | kFar32)) == kNear32) {
       near_words64(T.pre32[slot], T.pre64 + slot, T.nrm32[slot],
                    T.suf32p + (size_t)u * L.npairs, T.suf64 + (size_t)u * L.ns, j0,
                    j0 + C->sz[l], V, t, img);
