@@ -110,7 +110,6 @@ struct ExactTally {
 
 // Queue entry: prefix slot (bits 0-31), suffix letter (32-33), point (34-63).
 constexpr uint32_t kPendCap = 127;
-constexpr int kExactLanes = 24;  // lanes from which on each takes its own prefix's exact words
 constexpr int kDone = -2;  // pixel of a lane whose remaining words are left to the exact map
 
 // The n words of a warp's queue.  Out of line: it runs for about one word in
@@ -133,16 +132,18 @@ __device__ __noinline__ ExactTally exact_queue(const ExactCtx* C, const unsigned
 
 // Words [j0, j1) of each lane with `live` by the exact map (prefixes the filter does
 // not serve: direct form, out of range; words past a full queue): the lanes'
-// prefixes one after the other, split over the whole warp, or, where most lanes
-// have one (a view or generators out of the filter's range), each lane its own,
-// whose runs then are as long as in a render without a filter.  Near-cusp group,
+// prefixes one after the other, split over the whole warp, or, where that takes
+// about as many steps (most lanes have one, as in a view or with generators out of
+// the filter's range, or there are few words), each lane its own, whose runs then
+// are as long as in a render without a filter.  Near-cusp group,
 // 13 letters, 900 x 800, half width 1e-14: FP64 141 -> 94 us, double-float 146 -> 98;
 // 1e15, all words in one pixel: 1413 -> 269 and 1477 -> 280.
 template <int PREC>
 __device__ __noinline__ ExactTally exact_words(const ExactCtx* C, bool live, uint32_t slot,
                                                uint32_t u, uint32_t j0, uint32_t j1) {
   unsigned b = __ballot_sync(0xFFFFFFFFu, live);
-  const bool apart = __popc(b) >= kExactLanes;
+  const uint32_t most = __reduce_max_sync(0xFFFFFFFFu, live ? j1 - j0 : 0u);
+  const bool apart = 4u * __popc(b) * ((most + 31u) / 32u) >= 3u * most;
   Tally t;
   for (b = apart ? 1u : b; b; b &= b - 1u) {
     const int k = __ffs(b) - 1;
