@@ -353,15 +353,24 @@ struct WordWarp {
                 fabsf(Y + __uint_as_float((uint32_t)B.AY)) < B.hy) {
               ++run;
             } else if (j < ns && pix != kDone) {
-              add(pix, run, img);
-              run = open_box(pf, V, X, Y, B, pix) ? 1u : 0u;
-              if (!run) {
+              // (a box may end within its pixel: the run goes on)
+              const int was = pix;
+              const bool sure = open_box(pf, V, X, Y, B, pix);
+              if (pix != was) {
+                add(was, run, img);
+                run = 0u;
+              }
+              if (sure) {
+                ++run;
+              } else {
                 const uint32_t k = atomicAdd(&Q->n, 1u);
                 if (k < kPendCap) {
                   Q->e[k] = (unsigned long long)slot | ((unsigned long long)u << 32) |
                             ((unsigned long long)j << 34);
                 } else {  // full: the rest of this lane's words by the exact map
                   Q->over[lane] = j;
+                  add(pix, run, img);
+                  run = 0u;
                   pix = kDone;
                   B.hx = B.hy = __int_as_float(0x7F800000);
                 }
