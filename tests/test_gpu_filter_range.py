@@ -35,6 +35,8 @@ def params(kl, prec, d, half, plen=0, W=300, H=260, flat=1.0):  # noqa: F811
     (13, 1e15, 4, 1.0),    # 27 prefixes of a letter: a lane each, five lanes idle
     (11, 1.3, 4, 3e7),     # pixels far wider than high
     (12, 1e-6, 5, 1.0),    # in range, nothing certified: full queues
+    (12, 2000.0, 0, 1.0),  # the limit set well inside one pixel, in range
+    (12, 60.0, 0, 1.0),    # in a few pixels
     (8, 1e-13, 0, 1.0),    # one word to a prefix and letter
     (9, 1e-13, 7, 1.0),    # three
 ])
